@@ -40,19 +40,19 @@ def listed():
     large = (700, *recipe(700))
     return [
         # the smallest call: W at one frequency of the tiny molecule, all launches and latency
-        sized("screen", *tiny, prec="bf16x3", freqs=1, rhs=1, name="screen tiny, 1 frequency"),
+        sized("screen", *tiny, prec="bf16x3", freqs=1, rhs=1, name="screen tiny 1 frequency"),
         # a chunk of residue frequencies with a right-hand side per core: the loop of every self-energy grid
-        sized("screen", *benzene, prec="bf16x3", freqs=64, rhs=6, name="screen benzene, 64"),
+        sized("screen", *benzene, prec="bf16x3", freqs=64, rhs=6, name="screen benzene 64"),
         # few frequencies of a large molecule: one QP iterate, a probe of W at chosen points
-        sized("screen", *large, prec="bf16x3", freqs=8, rhs=12, name="screen 700 states, 8"),
+        sized("screen", *large, prec="bf16x3", freqs=8, rhs=12, name="screen 700 states 8"),
         # the largest polarizabilities, read back whole
-        sized("chi0", *pentacene, prec="bf16x3", freqs=2, name="chi0 pentacene, 2"),
+        sized("chi0", *pentacene, prec="bf16x3", freqs=2, name="chi0 pentacene 2"),
         # the G0W0 self-energy of a small molecule on its whole satellite window, one dielectric build per residue
-        sized("sigma", *tiny, prec="bf16x3", points=400, name="sigma tiny, 400 points"),
+        sized("sigma", *tiny, prec="bf16x3", points=400, name="sigma tiny 400 points"),
         # the same grid in the mode that checks the others
         sized("sigma", *tiny, prec="fp64", points=400, name="sigma tiny fp64"),
         # FP64 check of W at a few frequencies of a middle-sized molecule
-        sized("screen", *benzene, prec="fp64", freqs=8, rhs=6, name="screen benzene fp64, 8"),
+        sized("screen", *benzene, prec="fp64", freqs=8, rhs=6, name="screen benzene fp64 8"),
         # quasiparticle energies of a molecule just received: load, imaginary-axis table, secant iteration
         sized("qp", *benzene, prec="bf16x3", name="qp benzene"),
         # spectrum requests as the server runs them: load into a resident context, plan, step, results
