@@ -11,39 +11,243 @@
 // X_j = dt sum_k g_k e^{2 pi i jk/n}, A_j = Re X_j / pi on nu_j = 2 pi j/(n dt).
 // The sum over k is a batched radix-2 Stockham FFT in FP64 (Stockham autosort form as in
 // E. Bainville, "OpenCL Fast Fourier Transform", 2010), one pass per kernel.
+#include <algorithm>
+
 #include "gwc_internal.h"
 
 namespace gwc {
 
 namespace {
 
-// coef[c][j] = q_j beta_j / w_j^2 with trapezoid weights q_j of the per-core grid.
-__global__ void cumulant_coef_kernel(const double* __restrict__ omega_rel, int n_w, const double* __restrict__ im_sigma,
-                                     int n_core, double* __restrict__ coef) {
-  int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= n_core * n_w) return;
-  int c = t / n_w, j = t % n_w;
-  const double* w = omega_rel + (size_t)c * n_w;
-  double q = 0.0;
-  if (j > 0) q += 0.5 * (w[j] - w[j - 1]);
-  if (j < n_w - 1) q += 0.5 * (w[j + 1] - w[j]);
-  double wj = w[j];
-  double beta = fabs(im_sigma[t]) * (1.0 / 3.14159265358979323846);
-  coef[t] = wj == 0.0 ? 0.0 : q * beta / (wj * wj);
+// ---- C~(t) on blocks of times ---------------------------------------------------------------------
+// C~ is band-limited by its grid (|w_j| <= w_max), and the times are far denser than its Nyquist step (30 eV
+// windows: w_max dt = 0.03 at n_t = 2^16, t_max = 2000). So on a block of B consecutive times, t = t_b + h s with
+// |s| <= 1 and h = B dt / 2, sum_j c_j e^{-i w_j t} is a polynomial of degree 31 in s to FP64 rounding as long as
+// w_max h <= 8 (the interpolation error of e^{-i x s} at 32 Chebyshev nodes is at most 2 J_32(x), 9e-17 at x = 8).
+// Its values at the 32 nodes +-s_m cost 2 FMAs per (node, j) (E_j cos and E_j sin of the 16 positive nodes,
+// E_j = c_j e^{-i w_j t_b}), the Chebyshev coefficients a 16 x 16 cosine transform per parity, and every time one
+// 32-term Chebyshev sum: 100 + 48 FMAs per time instead of 6 N_w at N_w = 800, B = 512. FP64 runs at 1/64 of the
+// FP32 rate here, so the FP64 instruction count is what bounds the path. Measured (n_t = 2^16), the whole spectrum with the direct
+// sum below and with this: 6.66 and 0.164 ms for one core at 400 points, 26.5 and 0.935 ms for 22 cores.
+constexpr int NP = 32;       // Chebyshev nodes of a block, NH of them positive
+constexpr int NH = NP / 2;
+constexpr int MAXB = 1024;   // times per block, a power of two in NP .. MAXB
+constexpr int MAXG = 4;      // consecutive blocks of one work item
+constexpr int CT = 256;      // threads
+
+// Times per block for core c's grid: the largest power of two with w_max B dt / 2 <= 8; 0 where not even NP times fit
+// (a grid beyond w_max dt = 1/2, or one that is not finite): that core takes the direct sum. Every thread gets it.
+__device__ int block_times(const double* __restrict__ w, int n_w, int n_t, double dt) {
+  __shared__ double wm[32];
+  double m = 0.0;
+  bool fine = true;
+  for (int j = threadIdx.x; j < n_w; j += blockDim.x) {
+    const double a = fabs(w[j]);
+    fine = fine && a < 1e300;  // false for infinities and NaN
+    m = fmax(m, a);
+  }
+  if (!fine) m = 1e300;
+  for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+  if ((threadIdx.x & 31) == 0) wm[threadIdx.x >> 5] = m;
+  __syncthreads();
+  m = 0.0;
+  for (int k = 0; k < (int)(blockDim.x >> 5); ++k) m = fmax(m, wm[k]);
+  int b = 0;
+  for (int t = NP; t <= MAXB && t <= n_t && m * dt * (0.5 * t) <= 8.0; t <<= 1) b = t;
+  return b;
 }
 
-// g[c][k] = w_k exp(C~(t_k) - eta t_k), C~ summed over the grid in FP64. Each thread takes KT consecutive
-// times: per grid point one sincos at its first time and one for the step w_j dt, then the phase advances
-// by that rotation (FP64 sincos runs at the FP64 rate, 1/64 of FP32 on this part; the rotation drifts by
-// ~KT ulp over a block).
+// coef[c][j] = q_j beta_j / w_j^2 with trapezoid weights q_j of the per-core grid, and (tab given, core on blocks)
+// tab[c][j][m] = cos(w_j h s_m), tab[c][j][NH + m] = sin(w_j h s_m), s_m = cos(pi (2 m + 1) / (2 NP)).
+__global__ void __launch_bounds__(CT) cumulant_coef_kernel(const double* __restrict__ omega_rel, int n_w,
+                                                            const double* __restrict__ im_sigma, int n_t, double dt,
+                                                            double* __restrict__ coef, double* __restrict__ tab) {
+  const int c = blockIdx.y;
+  const double* w = omega_rel + (size_t)c * n_w;
+  const int b = tab ? block_times(w, n_w, n_t, dt) : 0;
+  const int e = blockIdx.x * CT + threadIdx.x, j = e / NH, m = e % NH;
+  if (j >= n_w) return;
+  const double wj = w[j];
+  if (m == 0) {
+    double q = 0.0;
+    if (j > 0) q += 0.5 * (w[j] - w[j - 1]);
+    if (j < n_w - 1) q += 0.5 * (w[j + 1] - w[j]);
+    const double beta = fabs(im_sigma[(size_t)c * n_w + j]) * (1.0 / 3.14159265358979323846);
+    coef[(size_t)c * n_w + j] = wj == 0.0 ? 0.0 : q * beta / (wj * wj);
+  }
+  if (b == 0) return;
+  double sn, cs;
+  sincos(wj * ((0.5 * b * dt) * cospi((2 * m + 1) * (0.5 / NP))), &sn, &cs);
+  double* o = tab + ((size_t)c * n_w + j) * NP;
+  o[m] = cs;
+  o[NH + m] = sn;
+}
+
+// One work item: G consecutive blocks from block b0 of core c (all of its times).
+template <int G>
+__device__ void cumulant_blocks(const double* __restrict__ w, const double* __restrict__ coef, const double* __restrict__ tab,
+                                int n_w, int B, int b0, double dt, double eta, double2 (*es)[CT] /*[MAXG][CT]*/,
+                                double2 (*cf)[NP] /*[MAXG][NP]*/, const double* cosn, double* s0sh, double2* __restrict__ g) {
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const double step = B * dt, tc = dt * ((double)b0 * B + 0.5 * (B - 1));  // centre of the first block
+  double ar[G], ai[G];
+#pragma unroll
+  for (int u = 0; u < G; ++u) ar[u] = ai[u] = 0.0;
+  double s0 = 0.0;
+  for (int j0 = 0; j0 < n_w; j0 += CT) {
+    const int j = j0 + tid;
+    double2 e = make_double2(0.0, 0.0), r = make_double2(1.0, 0.0);
+    if (j < n_w) {
+      const double cj = coef[j];
+      if (cj != 0.0) {
+        double sn, cs;
+        sincos(w[j] * tc, &sn, &cs);
+        e = make_double2(cj * cs, -cj * sn);
+        if (G > 1) {
+          sincos(w[j] * step, &sn, &cs);
+          r = make_double2(cs, -sn);
+        }
+      }
+      s0 += cj;
+    }
+    __syncthreads();  // the previous chunk (or item) has been read
+#pragma unroll
+    for (int u = 0; u < G; ++u) {
+      es[u][tid] = e;
+      if (u + 1 < G) e = make_double2(e.x * r.x - e.y * r.y, e.x * r.y + e.y * r.x);
+    }
+    __syncthreads();
+    const int jn = min(CT, n_w - j0);
+    const double* t = tab + (size_t)j0 * NP + lane;
+#pragma unroll 4
+    for (int q = warp; q < jn; q += CT / 32) {
+      const double v = t[(size_t)q * NP];
+#pragma unroll
+      for (int u = 0; u < G; ++u) {
+        const double2 x = es[u][q];
+        ar[u] = fma(x.x, v, ar[u]);
+        ai[u] = fma(x.y, v, ai[u]);
+      }
+    }
+  }
+  // sums over the warps (es holds them), then the node values and sum_j c_j
+  __syncthreads();
+  double2* part = &es[0][0];  // [warp][u][node]
+#pragma unroll
+  for (int u = 0; u < G; ++u) part[(warp * G + u) * 32 + lane] = make_double2(ar[u], ai[u]);
+  for (int o = 16; o > 0; o >>= 1) s0 += __shfl_down_sync(0xffffffffu, s0, o);
+  if (lane == 0) s0sh[warp] = s0;
+  __syncthreads();
+  for (int e = tid; e < G * 32; e += CT) {
+    double2 a = part[e];
+#pragma unroll
+    for (int k = 1; k < CT / 32; ++k) {
+      const double2 x = part[k * G * 32 + e];
+      a.x += x.x;
+      a.y += x.y;
+    }
+    part[e] = a;  // read by this thread alone so far
+  }
+  __syncthreads();
+  // Chebyshev coefficients: even ones from E cos, odd ones from -i E sin
+  for (int e = tid; e < G * NP; e += CT) {
+    const int u = e / NP, p = e % NP;
+    const double2* v = part + u * 32 + (p & 1) * NH;
+    double2 a = make_double2(0.0, 0.0);
+#pragma unroll
+    for (int m = 0; m < NH; ++m) {
+      const double k = cosn[(p * (2 * m + 1)) & (4 * NP - 1)];
+      a.x = fma(v[m].x, k, a.x);
+      a.y = fma(v[m].y, k, a.y);
+    }
+    const double f = p == 0 ? 2.0 / NP : 4.0 / NP;
+    cf[u][p] = (p & 1) ? make_double2(f * a.y, -f * a.x) : make_double2(f * a.x, f * a.y);
+  }
+  double sum = 0.0;
+#pragma unroll
+  for (int k = 0; k < CT / 32; ++k) sum += s0sh[k];
+  __syncthreads();
+  for (int q = tid; q < B / 2; q += CT) {  // the times at +-s of every block
+    const double s = (2 * q + 1) / (double)B;
+    double t0 = 1.0, t1 = s;
+    double er[G], ei[G], dr[G], di[G];  // even and odd sums
+#pragma unroll
+    for (int u = 0; u < G; ++u) er[u] = ei[u] = dr[u] = di[u] = 0.0;
+#pragma unroll 4
+    for (int p = 0; p < NP; p += 2) {
+#pragma unroll
+      for (int u = 0; u < G; ++u) {
+        const double2 x = cf[u][p], y = cf[u][p + 1];
+        er[u] = fma(x.x, t0, er[u]);
+        ei[u] = fma(x.y, t0, ei[u]);
+        dr[u] = fma(y.x, t1, dr[u]);
+        di[u] = fma(y.y, t1, di[u]);
+      }
+      t0 = fma(2.0 * s, t1, -t0);
+      t1 = fma(2.0 * s, t0, -t1);
+    }
+#pragma unroll
+    for (int u = 0; u < G; ++u) {
+      const int kc = (b0 + u) * B + B / 2;
+#pragma unroll
+      for (int side = 0; side < 2; ++side) {
+        const int k = side ? kc - 1 - q : kc + q;
+        const double re = (side ? er[u] - dr[u] : er[u] + dr[u]) - sum, im = side ? ei[u] - di[u] : ei[u] + di[u];
+        const double mag = exp(re - eta * (dt * k)) * (k == 0 ? 0.5 : 1.0);
+        double sn, cs;
+        sincos(im, &sn, &cs);
+        g[k] = make_double2(mag * cs, mag * sn);
+      }
+    }
+  }
+}
+
+// g[c][k] = w_k exp(C~(t_k) - eta t_k), w_0 = 1/2, for the cores whose grid fits the blocks. gridDim.y = cores; an item is G
+// consecutive blocks (the rotation e^{-i w_j B dt} replaces a sincos per block and j), G the largest of 4, 2, 1 that
+// still gives four items per SM.
+__global__ void __launch_bounds__(CT) cumulant_block_kernel(const double* __restrict__ omega_rel, int n_w,
+                                                             const double* __restrict__ coef, const double* __restrict__ tab,
+                                                             int n_t, double dt, double eta, int n_sm, double2* __restrict__ g) {
+  __shared__ double2 es[MAXG][CT];
+  __shared__ double2 cf[MAXG][NP];
+  __shared__ double cosn[4 * NP];  // cos(pi k / (2 NP))
+  __shared__ double s0sh[CT / 32];
+  static_assert((CT / 32) * 32 <= CT, "the warps' partial sums fit in es");
+  const int c = blockIdx.y;
+  const double* w = omega_rel + (size_t)c * n_w;
+  const int B = block_times(w, n_w, n_t, dt);
+  if (B == 0) return;
+  if (threadIdx.x < 4 * NP) cosn[threadIdx.x] = cospi(threadIdx.x * (0.5 / NP));
+  __syncthreads();
+  const int nb = n_t / B;
+  const double* k = coef + (size_t)c * n_w;
+  const double* t = tab + (size_t)c * n_w * NP;
+  double2* o = g + (size_t)c * n_t;
+  const long long all = (long long)nb * gridDim.y, want = 4LL * n_sm;
+  if (nb >= 4 && all / 4 >= want) {
+    for (int b = 4 * blockIdx.x; b < nb; b += 4 * gridDim.x)
+      cumulant_blocks<4>(w, k, t, n_w, B, b, dt, eta, es, cf, cosn, s0sh, o);
+  } else if (nb >= 2 && all / 2 >= want) {
+    for (int b = 2 * blockIdx.x; b < nb; b += 2 * gridDim.x)
+      cumulant_blocks<2>(w, k, t, n_w, B, b, dt, eta, es, cf, cosn, s0sh, o);
+  } else {
+    for (int b = blockIdx.x; b < nb; b += gridDim.x)
+      cumulant_blocks<1>(w, k, t, n_w, B, b, dt, eta, es, cf, cosn, s0sh, o);
+  }
+}
+
+// The direct sum over the grid, for the cores whose grid does not fit the blocks (all of them without `blocks`). Each thread
+// takes KT consecutive times: per grid point one sincos at its first time and one for the step w_j dt, then the phase
+// advances by that rotation (the rotation drifts by ~KT ulp over a block).
 constexpr int KT = 32;
 
 __global__ void cumulant_time_kernel(const double* __restrict__ omega_rel, int n_w, const double* __restrict__ coef,
-                                     int n_core, int n_t, double dt, double eta, double2* __restrict__ g) {
+                                     int n_core, int n_t, double dt, double eta, int blocks, double2* __restrict__ g) {
   extern __shared__ double sh[];  // [2][n_w]
   double* sw = sh;
   double* sc = sh + n_w;
   const int c = blockIdx.y;
+  if (blocks && block_times(omega_rel + (size_t)c * n_w, n_w, n_t, dt) > 0) return;
   for (int j = threadIdx.x; j < n_w; j += blockDim.x) {
     sw[j] = omega_rel[(size_t)c * n_w + j];
     sc[j] = coef[(size_t)c * n_w + j];
@@ -122,19 +326,24 @@ __global__ void spectrum_out_kernel(const double2* __restrict__ X, int n, int n_
 
 int launch_cumulant_spectrum(const double* omega_rel, int n_w, const double* im_sigma, int n_core, int n_t, double t_max,
                              double eta, double* work_a, double* work_b, double* coef, double* twiddle, double* a_out,
-                             double* nu_out, cudaStream_t s) {
+                             double* nu_out, double* table, int n_sm, cudaStream_t s) {
   int launches = 0;
   const double dt = t_max / n_t;
-  int tot = n_core * n_w;
-  cumulant_coef_kernel<<<(tot + 255) / 256, 256, 0, s>>>(omega_rel, n_w, im_sigma, n_core, coef);
+  cumulant_coef_kernel<<<dim3((unsigned)(((long long)n_w * NH + CT - 1) / CT), n_core), CT, 0, s>>>(omega_rel, n_w, im_sigma,
+                                                                                                    n_t, dt, coef, table);
   ++launches;
+  if (table) {
+    const int per = std::max(1, std::min(n_t / NP, (6 * n_sm + n_core - 1) / n_core));
+    cumulant_block_kernel<<<dim3(per, n_core), CT, 0, s>>>(omega_rel, n_w, coef, table, n_t, dt, eta, n_sm, (double2*)work_a);
+    ++launches;
+  }
   size_t sm = sizeof(double) * 2 * (size_t)n_w;
   if (sm > 48 * 1024) {
     if (cudaFuncSetAttribute(cumulant_time_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) != cudaSuccess)
       return -1;
   }
   dim3 g((n_t + 256 * KT - 1) / (256 * KT), n_core);
-  cumulant_time_kernel<<<g, 256, sm, s>>>(omega_rel, n_w, coef, n_core, n_t, dt, eta, (double2*)work_a);
+  cumulant_time_kernel<<<g, 256, sm, s>>>(omega_rel, n_w, coef, n_core, n_t, dt, eta, table ? 1 : 0, (double2*)work_a);
   ++launches;
   twiddle_kernel<<<(n_t / 2 + 255) / 256, 256, 0, s>>>(n_t, (double2*)twiddle);
   ++launches;

@@ -631,7 +631,7 @@ gwc_status gwc_workspace_bytes(const gwc_system* sys, const gwc_options* opt, in
   int batch = opt->batch > 0 ? opt->batch : 64;
   size_t b = resident_bytes(sys, opt, z) + (size_t)batch * per_matrix_bytes(sys, z);
   b += (size_t)n_omega * sys->n_states * (4 + 4 + 8 + 16 + 8 + 4 * sys->n_core) + (size_t)n_omega * sys->n_occ * sys->n_core * 16;
-  b += (size_t)sys->n_core * opt->n_t * 32 + (size_t)opt->n_t * 8;
+  b += (size_t)sys->n_core * opt->n_t * 32 + (size_t)opt->n_t * 8 + (size_t)n_omega * sys->n_core * 8 * (1 + kCumulantTable);
   *bytes = b;
   return GWC_OK;
 }
@@ -1227,11 +1227,12 @@ gwc_status gwc_cumulant_spectrum(gwc_ctx* ctx, const double* omega_rel, int n_om
     ctx->cw_cap = nc * nt * 2;
   }
   if (nc * (size_t)n_omega > ctx->coef_cap) {
-    TRY(dalloc(ctx, &ctx->d_coef, nc * (size_t)n_omega));
+    TRY(dalloc(ctx, &ctx->d_coef, nc * (size_t)n_omega * (1 + kCumulantTable)));
     ctx->coef_cap = nc * (size_t)n_omega;
   }
   LAUNCH(launch_cumulant_spectrum(omega_rel, n_omega, im_sigma, (int)nc, (int)nt, ctx->opt.t_max, ctx->opt.eta,
-                                  ctx->d_cw_a, ctx->d_cw_b, ctx->d_coef, ctx->d_tw, a_out, nu_out, st));
+                                  ctx->d_cw_a, ctx->d_cw_b, ctx->d_coef, ctx->d_tw, a_out, nu_out,
+                                  ctx->d_coef + ctx->coef_cap, ctx->n_sm, st));
   return check_stream_error(ctx);
 }
 
@@ -1411,7 +1412,7 @@ gwc_status gwc_request_plan(gwc_ctx* ctx, const double* omega_rel, int n_omega, 
     ctx->cw_cap = nc * nt * 2;
   }
   if ((size_t)nc * n_omega > ctx->coef_cap) {
-    TRY(dalloc(ctx, &ctx->d_coef, (size_t)nc * n_omega));
+    TRY(dalloc(ctx, &ctx->d_coef, (size_t)nc * n_omega * (1 + kCumulantTable)));
     ctx->coef_cap = (size_t)nc * n_omega;
   }
   CU(cudaMemcpyAsync(ctx->d_req_wrel, wrel.data(), sizeof(double) * wrel.size(), cudaMemcpyHostToDevice, st));
@@ -1441,7 +1442,7 @@ gwc_status gwc_request_step(gwc_ctx* ctx, void* stream) {
                             ctx->d_req_pair_of, ctx->d_req_w, ctx->d_req_im, st));
   LAUNCH(launch_cumulant_spectrum(ctx->d_req_wrel, ctx->req_n_omega, ctx->d_req_im, nc, ctx->opt.n_t, ctx->opt.t_max,
                                   ctx->opt.eta, ctx->d_cw_a, ctx->d_cw_b, ctx->d_coef, ctx->d_tw, ctx->d_req_a,
-                                  ctx->d_req_nu, st));
+                                  ctx->d_req_nu, ctx->d_coef + ctx->coef_cap, ctx->n_sm, st));
   return check_stream_error(ctx);
 }
 
@@ -1845,7 +1846,8 @@ gwc_status enqueue_grouped_step(gwc_ctx* const* ctxs, int n, const GroupedPlan& 
     BCU(launch_request_dec(c->d_eps, c->d_core_idx, c->n_core, c->eps_f, c->d_req_wrel, c->req_n_omega, c->d_req_pair_of,
                            c->d_req_w, c->d_req_im, st));
     BCU(launch_cumulant_spectrum(c->d_req_wrel, c->req_n_omega, c->d_req_im, c->n_core, c->opt.n_t, c->opt.t_max,
-                                 c->opt.eta, c->d_cw_a, c->d_cw_b, c->d_coef, c->d_tw, c->d_req_a, c->d_req_nu, st));
+                                 c->opt.eta, c->d_cw_a, c->d_cw_b, c->d_coef, c->d_tw, c->d_req_a, c->d_req_nu,
+                                 c->d_coef + c->coef_cap, c->n_sm, st));
   }
   return GWC_OK;
 }

@@ -276,11 +276,14 @@ int launch_gdh_spectrum(const double* eps, const int* core_idx, int n_core, cons
 int launch_request_dec(const double* eps, const int* core_idx, int n_core, double eps_f, const double* omega_rel, int n_w,
                        const int* pair_of, const double* wpair, double* im, cudaStream_t s);
 
-// Cumulant + FFT; see cumulant.cu
+// Cumulant + FFT; see cumulant.cu. `table`: kCumulantTable doubles per (core, grid point), or null (every core then
+// takes the direct sum over the grid).
+constexpr int kCumulantTable = 32;
 int launch_cumulant_spectrum(const double* omega_rel, int n_w, const double* im_sigma, int n_core, int n_t,
                              double t_max, double eta, double* work_a /*[n_core][n_t][2]*/,
                              double* work_b /*[n_core][n_t][2]*/, double* coef /*[n_core][n_w]*/,
-                             double* twiddle /*[n_t/2][2]*/, double* a_out, double* nu_out, cudaStream_t s);
+                             double* twiddle /*[n_t/2][2]*/, double* a_out, double* nu_out, double* table, int n_sm,
+                             cudaStream_t s);
 
 // Sets the message returned by gwc_last_error(NULL) (calls without a context).
 void set_noctx_error(const char* msg);

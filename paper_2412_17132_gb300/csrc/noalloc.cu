@@ -111,8 +111,14 @@ extern "C" gwc_status gwc_cumulant_spectrum_noalloc(const double* omega_rel, int
   double* work_b = reinterpret_cast<double*>(base + kMaxWork);
   double* twiddle = reinterpret_cast<double*>(base + 2 * kMaxWork);
   double* coef = reinterpret_cast<double*>(base + 2 * kMaxWork + kMaxTwiddle);
+  // the cumulant's node table lies in the second FFT buffer, which the first FFT pass overwrites; a grid whose table is
+  // larger (n_core * n_omega > 2^14) takes the direct sum
+  double* table = (long long)n_core * n_omega * gwc::kCumulantTable <= 2LL * kMaxWork ? work_b : nullptr;
+  int dev = 0, n_sm = 1;
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    n_sm = 1;
   int n = gwc::launch_cumulant_spectrum(omega_rel, n_omega, im_sigma, n_core, n_t, t_max, eta, work_a, work_b, coef,
-                                        twiddle, a_out, nu_out, static_cast<cudaStream_t>(stream));
+                                        twiddle, a_out, nu_out, table, n_sm, static_cast<cudaStream_t>(stream));
   if (n < 0) {
     gwc::set_noctx_error(cudaGetErrorString(cudaGetLastError()));
     return GWC_ERR_CUDA;
