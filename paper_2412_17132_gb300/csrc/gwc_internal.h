@@ -140,8 +140,9 @@ int chi0_group_fill(void* dst, bool split3, const __nv_bfloat16* o_hi, const __n
                     const int* active, bool out64, int item0);
 int launch_chi0_tc_grouped(const void* d_groups, int n_groups, int n_items, bool complex_out, int grid, unsigned* status,
                            unsigned long long wait_ns, cudaStream_t s);
-// Split factorisation of F complex FP32 matrices (same layout and result as launch_ldlt_tc): per 64-column
-// panel one panel launch (one CTA per matrix) and one batched tensor-core trailing update over all matrices.
+// Split factorisation of F complex FP32 matrices (as launch_ldlt_tc, but nothing is kept above the diagonal): per
+// 64-column panel launches for the diagonal blocks, for the rows below them and for the tensor-core trailing
+// update, each over all matrices.
 // `work` holds ldlt_split_bytes(n, nrow, F) bytes. Returns the launches, -1 on a launch error or bad layout,
 // -2 if unsupported.
 size_t ldlt_split_bytes(int n, int nrow, int F);

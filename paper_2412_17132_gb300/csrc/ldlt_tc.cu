@@ -87,120 +87,305 @@ __device__ __forceinline__ void split4(const float (&v)[4], float4& hi, float4& 
   lo = make_float4(l[0], l[1], l[2], l[3]);
 }
 
-// ---- panel factorisation (warps 0-11) -----------------------------------------------------------
-// The kb x kb diagonal block (kb <= 64) is factored right-looking by all 384 threads, one barrier per
-// step, and the same kb steps form X = L^-1 of its unit lower factor. Every element (i, c <= i) of
-// the lower triangle is owned by one thread and held in a register: while c > j it is the Schur
-// complement entry, a_ic -= W_ij d_j^-1 W_cj, final after step c - 1 and then published to shared
-// memory as W_ic (d_i on the diagonal); from step c on the same register accumulates
-// X_ic -= l_ij X_jc (c <= j < i, X_jj = 1, l_ij = W_ij / d_j), published after step i - 1. Step j
-// reads only column j of W and row j of X, both published before the barrier that opens it.
-// The rows below then need no dependent chain: W_rows = A_rows X^T (a product over the panel
-// columns, X^T upper triangular) and L^T_rows = (W_rows D^-1)^T.
-struct PanelInv {
-  static constexpr int LDP = PW + 1;                  // padded row (conflict-free column access)
-  static constexpr int CH = 16 * (NT_PANEL / 32);     // 192 staged rows: 6 blocks of 32 x 2 group pairs
-  float2 (*dm)[LDP];   // [64][65] W below the diagonal, d on it
-  float2 (*xg)[PW];    // [64][64] xg[l][c] = X_cl (zero for c < l), 16-byte rows for broadcast loads
-  float2* dinv;        // [64] 1 / d
-  float2* dpiv;        // [64] d (a zero pivot replaced by 1)
-  float2 (*xr)[LDP];   // [64][65] X by rows while the block is factored ...
-  float2 (*ach)[LDP];  // [CH][65] ... then, aliased, the staged rows below the panel
-  static constexpr size_t bytes() {
-    return sizeof(float2) * ((size_t)PW * LDP + PW * PW + 2 * PW + (size_t)CH * LDP);
+// ---- diagonal blocks ---------------------------------------------------------------------------------
+// The kb x kb diagonal block (kb <= 64) and X = L^-1 of its unit lower factor, by NT threads. Every element (i, c) of the
+// lower triangle takes the right-looking updates in the order of the columns j,
+//     a_ic -= W_ij (d_j^-1 W_cj), j < c,     X_ic -= W_ij (d_j^-1 X_jc), c <= j < i (X_jj = 1).
+// What bounds the block is the chain of its 64 pivots (a reciprocal, two products and an exchange each), not its
+// arithmetic, so the columns go in four blocks of 16:
+//   pivots  one warp factors the 16 x 16 block in registers, two lanes per row;
+//   panel   a thread per row below and a thread per column of X finish the block's columns without any exchange;
+//   update  the next 16 x 16 block by all threads, then the rows below, for a and for X, in 2 x 4 tiles by the other warps
+//           while the first warp takes the next block's pivots.
+// The loops over j keep the current columns in front and shift: unrolled fully they were bound by instruction fetches. With one
+// CTA barrier per pivot and every d_j^-1 W_cj formed again by each thread that uses it a block
+// took 38 us; this takes 27 us (one to 152 matrices).
+constexpr int DB = 16;        // columns per block
+constexpr int LDB = 2 * DB;   // row of the in-block factors (the second half pads the shifted reads)
+constexpr int LDP = PW + 1;   // padded row (conflict-free column access)
+constexpr int LDM = PW + 2;   // row of the update's second operand (16-byte pairs)
+
+// Scratch of a diagonal block at byte offset `o` of the dynamic shared memory (addressed through the shared array itself:
+// pointers kept in a struct became generic loads)
+struct DiagSmem {
+  static constexpr int MJ = 0;                       // [16][66] d_j^-1 X_jc (columns c up to the block), d_j^-1 W_cj (beyond)
+  static constexpr int LB = MJ + DB * LDM;           // [16][32] d_j^-1 W_ij inside the block, (j, i)
+  static constexpr int WB = LB + DB * LDB;           // [16][32] W_ij inside the block, (j, i)
+  static constexpr int DINV = WB + DB * LDB;         // [64] 1 / d
+  static constexpr int DPIV = DINV + PW;             // [64] d (a zero pivot replaced by 1)
+  static constexpr int DM = DPIV + PW;               // [64][65] a, then W below the diagonal
+  static constexpr int XR = DM + PW * LDP;           // [64][65] X by rows
+  static constexpr int ELEMS = XR + PW * LDP;
+  uint32_t o;
+  __device__ __forceinline__ float2& at(int e) const {
+    extern __shared__ uint8_t smem_raw[];
+    return *reinterpret_cast<float2*>(smem_raw + o + e * 8);
   }
-  __device__ explicit PanelInv(void* base) {
-    float2* p = reinterpret_cast<float2*>(base);
-    dm = reinterpret_cast<float2(*)[LDP]>(p);
-    p += PW * LDP;
-    xg = reinterpret_cast<float2(*)[PW]>(p);
-    p += PW * PW;
-    dinv = p;
-    dpiv = p + PW;
-    p += 2 * PW;
-    xr = reinterpret_cast<float2(*)[LDP]>(p);
-    ach = reinterpret_cast<float2(*)[LDP]>(p);
+  __device__ __forceinline__ float4 pair(int e) const {  // two neighbours, e even
+    extern __shared__ uint8_t smem_raw[];
+    return *reinterpret_cast<const float4*>(smem_raw + o + e * 8);
   }
+  __device__ __forceinline__ float2& dm(int i, int c) const { return at(DM + i * LDP + c); }
+  __device__ __forceinline__ float2& xr(int i, int c) const { return at(XR + i * LDP + c); }
+  __device__ __forceinline__ float2& mj(int j, int c) const { return at(MJ + j * LDM + c); }
+  __device__ __forceinline__ float2& lb(int j, int i) const { return at(LB + j * LDB + i); }
+  __device__ __forceinline__ float2& wb(int j, int i) const { return at(WB + j * LDB + i); }
+  __device__ __forceinline__ float2& dinv(int j) const { return at(DINV + j); }
+  __device__ __forceinline__ float2& dpiv(int j) const { return at(DPIV + j); }
 };
-static_assert(PanelInv::bytes() <= (size_t)OPS_BYTES, "panel scratch fits in the operand buffers");
-static_assert(PW * PW <= PanelInv::CH * PanelInv::LDP, "X by rows fits in the staging rows");
 
-__device__ __forceinline__ void panel_sync() { grp_sync_n<NT_PANEL>(); }
+// products with their roundings written out, so that a factor has the same bits whichever thread forms it
+__device__ __forceinline__ float2 cmul_rn(float2 a, float2 b) {
+  return make_float2(__fmaf_rn(a.x, b.x, -__fmul_rn(a.y, b.y)), __fmaf_rn(a.y, b.x, __fmul_rn(a.x, b.y)));
+}
+__device__ __forceinline__ float cabs2_rn(float2 a) { return __fmaf_rn(a.x, a.x, __fmul_rn(a.y, a.y)); }
 
-// diagonal block [k0, k0 + kb): W / d / L^T stored to A; dinv and xg left in shared memory
-__device__ void factor_diag_block(float2* __restrict__ A, long long ldm, int k0, int kb, const PanelInv& ps,
-                                  int* sing) {
-  constexpr int MAXS = (PW * (PW + 1) / 2 + NT_PANEL - 1) / NT_PANEL;
-  const int tid = threadIdx.x;
-  panel_sync();  // the previous phase's use of the scratch is over
-  for (int e = tid; e < PW * PW; e += NT_PANEL) {
-    const int i = e >> 6, c = e & 63;
-    ps.dm[i][c] = (i < kb && c <= i) ? A[(long long)(k0 + i) * ldm + (k0 + c)] : make_float2(0.f, 0.f);
-    ps.xr[i][c] = make_float2(i == c ? 1.f : 0.f, 0.f);
-  }
-  panel_sync();
-  int si[MAXS], sc[MAXS];
-  float2 v[MAXS];
-  const int tot = kb * (kb + 1) / 2;
+__device__ __forceinline__ float2 shfl2(float2 v, int src) {
+  return make_float2(__shfl_sync(0xffffffffu, v.x, src), __shfl_sync(0xffffffffu, v.y, src));
+}
+
+// v[c] -= w m[c] for the columns c = 2 .. 15 beyond an even column 0 (m 16-byte aligned)
+__device__ __forceinline__ void cols_after_even(float2 (&v)[DB], float2 w, const DiagSmem& ds, int m) {
 #pragma unroll
-  for (int s = 0; s < MAXS; ++s) {
-    const int e = tid + s * NT_PANEL;
-    int i = -1, c = 0;
-    if (e < tot) {
-      i = (int)((sqrtf(8.f * (float)e + 1.f) - 1.f) * 0.5f);
-      while (i * (i + 1) / 2 > e) --i;
-      while ((i + 1) * (i + 2) / 2 <= e) ++i;
-      c = e - i * (i + 1) / 2;
-      v[s] = ps.dm[i][c];
-    } else {
-      v[s] = make_float2(0.f, 0.f);
-    }
-    si[s] = i;
-    sc[s] = c;
+  for (int c = 2; c < DB; c += 2) {
+    const float4 x = ds.pair(m + c);
+    v[c] = sfnms(w, make_float2(x.x, x.y), v[c]);
+    v[c + 1] = sfnms(w, make_float2(x.z, x.w), v[c + 1]);
   }
-  for (int j = 0; j < kb; ++j) {
-    float2 d = ps.dm[j][j];
-    const bool zero = fabsf(d.x) + fabsf(d.y) < 1e-30f;
+}
+
+// Pivots of the 16 x 16 block at j0 (its values in ds.dm) by one warp. Lanes i and 16 + i share row i: both carry the current pair
+// of columns (v0, v1), and each the further columns of its parity (f[k] = column 2 + 2k + h of the row, relative to the pair). Of the
+// reciprocal each half forms one part (one division instead of two in the chain), and the next pivot is formed by its own lane.
+__device__ __forceinline__ void diag_pivots(int j0, int w16, const DiagSmem& ds, int* sing) {
+  const int lane = threadIdx.x & 31, i = lane & 15, h = lane >> 4;
+  float2 v0 = ds.dm(j0 + i, j0), v1 = ds.dm(j0 + i, j0 + 1), f[DB / 2 - 1];
+#pragma unroll
+  for (int k = 0; k + 1 < DB / 2; ++k) f[k] = ds.dm(j0 + i, j0 + 2 + 2 * k + h);
+  bool zero;
+  float2 d = shfl2(v0, 0), inv;
+  auto pivot = [&] {
+    zero = fabsf(d.x) + fabsf(d.y) < 1e-30f;
     if (zero) d = make_float2(1.f, 0.f);
-    const float2 inv = sinv(d);
-    if (tid == 0) {
-      ps.dinv[j] = inv;
-      ps.dpiv[j] = d;
+    const float den = cabs2_rn(d);
+    const float q = __fdiv_rn(h ? -d.y : d.x, den), o = __shfl_xor_sync(0xffffffffu, q, 16);
+    inv = h ? make_float2(o, q) : make_float2(q, o);
+  };
+  pivot();
+  // one column: l = d^-1 w published, the next column `next` updated, its pivot and reciprocal started
+  auto column = [&](int j, float2 w, float2& next) {
+    if (lane == j) {
+      ds.dinv(j0 + j) = inv;
+      ds.dpiv(j0 + j) = d;
       if (zero) *sing = 1;
     }
+    const float2 l = cmul_rn(inv, w);
+    if (i > j && lane < w16) {
+      ds.dm(j0 + i, j0 + j) = w;
+      ds.wb(j, i) = w;
+      ds.lb(j, i) = l;
+    }
+    const float2 e = sfnms(w, l, next);  // the diagonal entry in lane j + 1
+    d = shfl2(e, j + 1);                 // (after the last column, a value that is not used)
+    next = sfnms(w, shfl2(l, j + 1), next);
+    pivot();
+    __syncwarp();
+  };
+#pragma unroll 1
+  for (int j = 0; j < w16; j += 2) {
+    const float2 o = make_float2(__shfl_xor_sync(0xffffffffu, f[0].x, 16), __shfl_xor_sync(0xffffffffu, f[0].y, 16));
+    float2 v2 = h ? o : f[0], v3 = h ? f[0] : o;
+    column(j, v0, v1);
+    {
+      const float4 x = ds.pair(DiagSmem::LB + j * LDB + j + 2);
+      v2 = sfnms(v0, make_float2(x.x, x.y), v2);
+      v3 = sfnms(v0, make_float2(x.z, x.w), v3);
 #pragma unroll
-    for (int s = 0; s < MAXS; ++s) {
-      const int i = si[s], c = sc[s];
-      if (i > j) {
-        const float2 wij = ps.dm[i][j];
-        if (c > j) {
-          v[s] = sfnms(wij, smul(inv, ps.dm[c][j]), v[s]);
-          if (c == j + 1) ps.dm[i][c] = v[s];
-        } else {
-          if (c == j) v[s] = make_float2(0.f, 0.f);
-          v[s] = sfnms(wij, smul(inv, ps.xr[j][c]), v[s]);
-          if (i == j + 1) ps.xr[i][c] = v[s];
+      for (int k = 1; k + 1 < DB / 2; ++k) f[k] = sfnms(v0, ds.lb(j, j + 2 + 2 * k + h), f[k]);
+    }
+    if (j + 1 >= w16) break;  // uniform
+    column(j + 1, v1, v2);
+    {
+      v3 = sfnms(v1, ds.lb(j + 1, j + 3), v3);
+#pragma unroll
+      for (int k = 1; k + 1 < DB / 2; ++k) f[k] = sfnms(v1, ds.lb(j + 1, j + 2 + 2 * k + h), f[k]);
+    }
+    v0 = v2;
+    v1 = v3;
+#pragma unroll
+    for (int k = 0; k + 2 < DB / 2; ++k) f[k] = f[k + 1];
+  }
+}
+
+// v[c] -= w m[c], c >= 1 beyond column 0 of an even pair (first) or c >= 2 beyond column 1 (second)
+__device__ __forceinline__ void panel_step(float2 (&v)[DB], float2 w, const DiagSmem& ds, int m, bool first) {
+  if (first) {
+    v[1] = sfnms(w, ds.at(m + 1), v[1]);
+  }
+  cols_after_even(v, w, ds, m);
+}
+
+// diagonal block [k0, k0 + kb): W and d stored to A (and L^T above the diagonal if `lt`); dinv and xr left in shared memory
+template <int NT>
+__device__ void factor_diag_block(float2* __restrict__ A, long long ldm, int k0, int kb, const DiagSmem& ds, int* sing, bool lt) {
+  static_assert(NT % 32 == 0 && NT >= DB * DB, "a thread per entry of a 16 x 16 block");
+  const int tid = threadIdx.x;
+  grp_sync_n<NT>();  // the previous phase's use of the scratch is over
+  constexpr int PT = (PW * PW + NT - 1) / NT;
+  for (int h = 0; h < PT; h += 8) {
+    float2 v[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const int e = tid + (h + q) * NT, i = e >> 6, c = e & 63;
+      v[q] = (i < kb && c <= i) ? A[(long long)(k0 + i) * ldm + (k0 + c)] : make_float2(0.f, 0.f);
+    }
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const int e = tid + (h + q) * NT, i = e >> 6, c = e & 63;
+      if (e < PW * PW) {
+        ds.dm(i, c) = v[q];
+        ds.xr(i, c) = make_float2(i == c ? 1.f : 0.f, 0.f);
+      }
+    }
+  }
+  grp_sync_n<NT>();
+  if (tid < 32) diag_pivots(0, min(DB, kb), ds, sing);
+  grp_sync_n<NT>();
+  for (int j0 = 0; j0 < kb; j0 += DB) {
+    const int w16 = min(DB, kb - j0), j1 = j0 + w16;
+    if (tid < kb - j1) {  // row i below the block: its 16 columns of W, and d^-1 W as the update's second operand
+      const int i = j1 + tid;
+      float2 v[DB];
+#pragma unroll
+      for (int c = 0; c < DB; ++c) v[c] = ds.dm(i, j0 + c);
+#pragma unroll 1
+      for (int j = 0; j < DB; j += 2) {
+        const float2 w0 = v[0];
+        panel_step(v, w0, ds, DiagSmem::LB + j * LDB + j, true);
+        const float2 w1 = v[1];
+        panel_step(v, w1, ds, DiagSmem::LB + (j + 1) * LDB + j, false);
+        ds.dm(i, j0 + j) = w0;
+        ds.dm(i, j0 + j + 1) = w1;
+        ds.mj(j, i) = cmul_rn(ds.dinv(j0 + j), w0);
+        ds.mj(j + 1, i) = cmul_rn(ds.dinv(j0 + j + 1), w1);
+#pragma unroll
+        for (int c = 0; c + 2 < DB; ++c) v[c] = v[c + 2];
+      }
+    } else if (tid >= 64 && tid < 64 + j1) {  // column c of X: its rows in the block (zero above the diagonal)
+      const int c = tid - 64;
+      float2 x[DB];
+#pragma unroll
+      for (int j = 0; j < DB; ++j) x[j] = ds.xr(j0 + j, c);
+#pragma unroll 1
+      for (int j = 0; j < w16; j += 2) {
+#pragma unroll
+        for (int s = 0; s < 2; ++s) {
+          if (j + s >= w16) break;
+          const bool on = j0 + j + s >= c;
+          const float2 xj = x[s], xs = on ? cmul_rn(ds.dinv(j0 + j + s), xj) : make_float2(0.f, 0.f);
+          ds.xr(j0 + j + s, c) = xj;
+          ds.mj(j + s, c) = xs;
+          if (on) {  // x_i -= W_ij (d_j^-1 x_j): the operands in the order of the update below
+            const int m = DiagSmem::WB + (j + s) * LDB + j;
+            if (s == 0) x[1] = sfnms(ds.at(m + 1), xs, x[1]);
+#pragma unroll
+            for (int i = 2; i < DB; i += 2) {
+              const float4 w = ds.pair(m + i);
+              x[i] = sfnms(make_float2(w.x, w.y), xs, x[i]);
+              x[i + 1] = sfnms(make_float2(w.z, w.w), xs, x[i + 1]);
+            }
+          }
+        }
+#pragma unroll
+        for (int i = 0; i + 2 < DB; ++i) x[i] = x[i + 2];
+      }
+    }
+    grp_sync_n<NT>();
+    const int nr = kb - j1;
+    if (nr <= 0) break;  // (below, j1 < kb: the block is full)
+    if (tid < DB * DB) {  // the next 16 x 16 block takes the 16 updates, an entry per thread
+      const int r = tid >> 4, c = tid & 15, i = j1 + r;
+      if (c <= r && i < kb) {
+        float2 v = ds.dm(i, j1 + c);
+#pragma unroll 8
+        for (int j = 0; j < DB; ++j) v = sfnms(ds.dm(i, j0 + j), ds.mj(j, j1 + c), v);
+        ds.dm(i, j1 + c) = v;
+      }
+    }
+    grp_sync_n<NT>();
+    if (tid < 32) {
+      diag_pivots(j1, min(DB, nr), ds, sing);
+    } else {
+      // rows below the block: a_ic (c beyond the block) and X_ic (c up to it); a thread's rows are r and r + tr
+      const int tr = (nr + 1) >> 1;
+      for (int e = tid - 32; e < tr * (PW / 4); e += NT - 32) {
+        const int r = e % tr, c0 = 4 * (e / tr), i0 = j1 + r, i1 = min(i0 + tr, kb - 1);
+        if (c0 > i1 || (c0 >= j1 && i1 < j1 + DB)) continue;  // above the diagonal, or the next 16 x 16 block
+        const bool x_side = c0 < j1;  // a tile lies on one side: j1 is a multiple of 4
+        const int t = (x_side ? DiagSmem::XR : DiagSmem::DM) + c0, t0 = t + i0 * LDP, t1 = t + i1 * LDP;
+        float2 v[2][4];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          v[0][c] = ds.at(t0 + c);
+          v[1][c] = ds.at(t1 + c);
+        }
+#pragma unroll 2
+        for (int j = 0; j < DB; ++j) {
+          const float2 w0 = ds.dm(i0, j0 + j), w1 = ds.dm(i1, j0 + j);
+          const float4 m0 = ds.pair(DiagSmem::MJ + j * LDM + c0);
+          const float4 m1 = ds.pair(DiagSmem::MJ + j * LDM + c0 + 2);
+          const float2 m[4] = {make_float2(m0.x, m0.y), make_float2(m0.z, m0.w), make_float2(m1.x, m1.y),
+                               make_float2(m1.z, m1.w)};
+#pragma unroll
+          for (int c = 0; c < 4; ++c) {
+            v[0][c] = sfnms(w0, m[c], v[0][c]);
+            v[1][c] = sfnms(w1, m[c], v[1][c]);
+          }
+        }
+        // (entries above the diagonal of a tile on it are not used; the next 16 x 16 block is the first warp's)
+        const bool s0 = x_side || i0 >= j1 + DB, s1 = i0 + tr < kb;
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          if (s0) ds.at(t0 + c) = v[0][c];
+          if (s1) ds.at(t1 + c) = v[1][c];
         }
       }
     }
-    panel_sync();
+    grp_sync_n<NT>();
   }
-  for (int e = tid; e < PW * PW; e += NT_PANEL) {
-    const int l = e >> 6, c = e & 63;
-    ps.xg[l][c] = (c >= l && c < kb) ? ps.xr[c][l] : make_float2(0.f, 0.f);
+  for (int e = tid; e < PW * PW; e += NT) {
+    const int i = e >> 6, c = e & 63;
+    if (i >= kb || c > i) continue;
+    const float2 w = c < i ? ds.dm(i, c) : ds.dpiv(i);
+    A[(long long)(k0 + i) * ldm + (k0 + c)] = w;
+    if (lt && c < i) A[(long long)(k0 + c) * ldm + (k0 + i)] = smul(w, ds.dinv(c));
   }
-  for (int e = tid; e < kb * kb; e += NT_PANEL) {
-    const int i = e / kb, c = e % kb;
-    if (c < i) {
-      const float2 w = ps.dm[i][c];
-      A[(long long)(k0 + i) * ldm + (k0 + c)] = w;
-      A[(long long)(k0 + c) * ldm + (k0 + i)] = smul(w, ps.dinv[c]);
-    } else if (c == i) {
-      A[(long long)(k0 + i) * ldm + (k0 + i)] = ps.dpiv[i];
-    }
-  }
-  panel_sync();  // xg, dinv complete; xr may be overwritten by the staged rows
 }
+
+// ---- panel factorisation of the one-CTA kernel (warps 0-11) --------------------------------------------
+// The diagonal block above, then the rows below without any dependent chain: W_rows = A_rows X^T (a product over the panel
+// columns, X^T upper triangular) and L^T_rows = (W_rows D^-1)^T.
+struct PanelInv {
+  static constexpr int CH = 16 * (NT_PANEL / 32);     // 192 staged rows: 6 blocks of 32 x 2 group pairs
+  float2 (*xg)[PW];    // [64][64] xg[l][c] = X_cl (zero for c < l), 16-byte rows for broadcast loads
+  DiagSmem ds;         // scratch of the diagonal block (1 / d stays) ...
+  float2* dinv;
+  float2 (*ach)[LDP];  // [CH][65] ... the staged rows below the panel after it (aliases dm and xr)
+  static constexpr size_t bytes() { return sizeof(float2) * (PW * PW + DiagSmem::DM + (size_t)CH * LDP); }
+  __device__ explicit PanelInv(uint8_t* base) {
+    extern __shared__ uint8_t smem_raw[];
+    float2* p = reinterpret_cast<float2*>(base);
+    xg = reinterpret_cast<float2(*)[PW]>(p);
+    p += PW * PW;
+    ds.o = smem_u32(p) - smem_u32(smem_raw);
+    dinv = p + DiagSmem::DINV;
+    ach = reinterpret_cast<float2(*)[LDP]>(p + DiagSmem::DM);
+  }
+};
+static_assert(PanelInv::bytes() <= (size_t)OPS_BYTES, "panel scratch fits in the operand buffers");
+static_assert(2 * PW <= PanelInv::CH, "the diagonal block fits in the staging rows");
+
+__device__ __forceinline__ void panel_sync() { grp_sync_n<NT_PANEL>(); }
 
 // One warp's share of a staged chunk: rows r0 .. r0 + 31 (one per lane), the 16 columns of group g,
 // w_c = sum_{l <= c} a_l X_cl in packed FP32 pairs (re and im of X per product), then W (row-major,
@@ -264,8 +449,16 @@ __device__ __forceinline__ void panel_rows_group(float2* __restrict__ A, int n, 
 __device__ void factor_panel_tc(float2* __restrict__ A, int n, int nrow, long long ldm, int k0, const PanelInv& ps,
                                 int* sing) {
   const int kb = min(PW, n - k0);
-  factor_diag_block(A, ldm, k0, kb, ps, sing);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  {
+    const DiagSmem ds = ps.ds;
+    factor_diag_block<NT_PANEL>(A, ldm, k0, kb, ds, sing, true);
+    for (int e = tid; e < PW * PW; e += NT_PANEL) {
+      const int l = e >> 6, c = e & 63;
+      ps.xg[l][c] = (c >= l && c < kb) ? ds.xr(c, l) : make_float2(0.f, 0.f);
+    }
+    panel_sync();  // xg, dinv complete; dm and xr may be overwritten by the staged rows
+  }
   const int r = 32 * (warp >> 1) + lane;
   const int g0 = (warp & 1) ? 1 : 0, g1 = (warp & 1) ? 2 : 3;
   for (int base = k0 + kb; base < nrow; base += PanelInv::CH) {
@@ -726,18 +919,18 @@ __global__ void __launch_bounds__(NT_TC, 1)
   ldlt_tc_matrix(G.mats + f * G.stride, G.n, G.nrow, G.ldm, status, wait_ns);
 }
 
-// ---- split factorisation: one panel launch and one batched tensor-core update per panel --------------
+// ---- split factorisation: per panel, launches over all matrices of the batch -------------------------
 // The kernel above gives each matrix one CTA for its whole factorisation, and its tensor phase waits on
 // the per-thread global loads of one SM (a 4500-wide matrix takes ~190 ms). Here every panel is three
 // launches over all matrices of the batch:
-//   ldlt_panel_kernel   the panel [k0, k0 + 64) of every matrix (one CTA each: factor_panel_tc);
-//   ldlt_planes_kernel  the panel's W columns (rows below it) and L rows (row k0 + l of the L^T stored above
-//                       the diagonal, the columns beyond the panel) as TF32 hi / lo planes, K-major;
+//   ldlt_diag_kernel    the 64 x 64 diagonal block and the inverse of its unit lower factor (one CTA per matrix);
+//   ldlt_rows_kernel    the rows below it (64 per CTA), with the panel's W columns and L rows as TF32 hi / lo
+//                       planes, K-major (L^T is not kept above the diagonal: only the planes feed the update);
 //   ldlt_update_kernel  C[i][j] -= sum_l W[i][l] L[j][l] over the trailing 128 x 64 tiles of every matrix,
 //                       one tile per CTA, two CTAs per SM: TMA-fed planes, the P and Q accumulators of the
 //                       one-CTA kernel, and the target tile staged through shared memory by TMA (128-byte
 //                       swizzle, clipped at column n and row nrow; the part of a diagonal tile above the
-//                       diagonal holds nothing yet and is overwritten when its own panel is factored).
+//                       diagonal holds nothing).
 // Panels go in pairs with a one-panel lookahead: panel p's update is first applied to panel p + 1's 64
 // columns only, panel p + 1 is factored, and then one rank-128 update (K = 128: both panels' planes side by
 // side) covers the trailing matrix, which is thus read and written once per two panels.
@@ -747,8 +940,11 @@ constexpr int UP_B = TN * 128;                   // one B plane chunk: 64 rows x
 constexpr int UP_STAGE = 4 * UP_A + 4 * UP_B;    // Ar, Ai, Ar_lo, Ai_lo | Lr, Li, Lr_lo, Li_lo: 96 KB
 constexpr int UP_SMEM = 1024 + UP_STAGE + 128;
 constexpr int UP_THREADS = 256;                  // warp 0 TMA, 1 MMA, 2 TMEM, 4-7 epilogue
-constexpr int PANEL_SCRATCH = (int)PanelInv::bytes();
-constexpr int PANEL_SMEM = 1024 + PANEL_SCRATCH + 64;
+constexpr int XD = PW * PW + PW;                 // X and 1 / d of a panel, per matrix
+constexpr int DIAG_THREADS = 256;
+constexpr int DIAG_SMEM = DiagSmem::ELEMS * (int)sizeof(float2);
+constexpr int ROWS_THREADS = 128;                // 64 rows x 64 columns per CTA
+constexpr int ROWS_SMEM = (XD + 64 * LDP) * (int)sizeof(float2);
 static_assert(TM * TN * 8 <= UP_STAGE, "the target tile fits in the stage");
 
 constexpr int KW = 2 * PW;  // K width of the planes: two panels
@@ -779,60 +975,124 @@ __device__ __forceinline__ void tma_store_3d(const CUtensorMap* tm, int x, int y
                : "memory");
 }
 
-__global__ void __launch_bounds__(NT_PANEL, 1)
-    ldlt_panel_kernel(float2* __restrict__ mats, int n, int nrow, long long ldm, long long stride, int k0,
-                      const int* __restrict__ active, unsigned* __restrict__ status) {
+// the diagonal block of panel k0 of every matrix (one CTA each); X = L^-1 as xg[l][c] = X_cl and 1 / d to `xd` for the rows below
+__global__ void __launch_bounds__(DIAG_THREADS)
+    ldlt_diag_kernel(float2* __restrict__ mats, int n, long long ldm, long long stride, int k0, const int* __restrict__ active,
+                     float2* __restrict__ xd, unsigned* __restrict__ status) {
   const int f = blockIdx.x;
   if (active && !active[f]) return;
-  extern __shared__ uint8_t smem_raw[];
-  uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-  const PanelInv ps(base);
-  int* sing = reinterpret_cast<int*>(base + PANEL_SCRATCH);
-  if (threadIdx.x == 0) *sing = 0;
-  __syncthreads();
-  factor_panel_tc(mats + f * stride, n, nrow, ldm, k0, ps, sing);
-  __syncthreads();
-  if (threadIdx.x == 0 && *sing) atomicOr(status, kStatSingular);
+  const DiagSmem ds{0};
+  __shared__ int sing;
+  if (threadIdx.x == 0) sing = 0;
+  const int kb = min(PW, n - k0);
+  factor_diag_block<DIAG_THREADS>(mats + f * stride, ldm, k0, kb, ds, &sing, false);
+  float2* o = xd + (size_t)f * XD;
+  for (int e = threadIdx.x; e < PW * PW; e += DIAG_THREADS) {
+    const int l = e >> 6, c = e & 63;
+    o[e] = (c >= l && c < kb) ? ds.xr(c, l) : make_float2(0.f, 0.f);
+  }
+  if (threadIdx.x < PW) o[PW * PW + threadIdx.x] = threadIdx.x < kb ? ds.dinv(threadIdx.x) : make_float2(0.f, 0.f);
+  if (threadIdx.x == 0 && sing) atomicOr(status, kStatSingular);
 }
 
-// blockIdx.y = matrix; blocks 0 .. nA-1: four rows i of W each; blocks nA ..: 32 columns j of L each
-__global__ void __launch_bounds__(256)
-    ldlt_planes_kernel(const float2* __restrict__ mats, int n, int nrow, long long ldm, long long stride, int k0, int koff,
-                       int nA, const int* __restrict__ active, float* __restrict__ ap, float* __restrict__ bp) {
+__device__ __forceinline__ void store_planes(float* __restrict__ o, size_t plane, const float2 (&v)[8]) {
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {
+    float re[4], im[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      re[e] = v[4 * q + e].x;
+      im[e] = v[4 * q + e].y;
+    }
+    float4 rh, rl, ih, il;
+    split4(re, rh, rl);
+    split4(im, ih, il);
+    *reinterpret_cast<float4*>(o + 4 * q) = rh;
+    *reinterpret_cast<float4*>(o + plane + 4 * q) = ih;
+    *reinterpret_cast<float4*>(o + 2 * plane + 4 * q) = rl;
+    *reinterpret_cast<float4*>(o + 3 * plane + 4 * q) = il;
+  }
+}
+
+// Rows below panel k0, 64 per CTA (blockIdx.x) of matrix blockIdx.y: W = A X^T, stored to A, and the TF32 hi / lo planes of W
+// (rows i) and of L = W D^-1 (the rows that are columns of the trailing matrix, j < n) that the update reads, K-major at K
+// column koff. Warp w takes the 32-row block w / 2 and the column groups {0, 3} or {1, 2} (equal work: the triangle of X).
+// The rows were the panel CTA's second half, 192 at a time on one SM per matrix (21 us each), and the planes a kernel
+// of their own: 8 matrices of N_aux 2450, panels and planes of a factorisation 7.1 ms, diagonal blocks and rows now 1.8 ms;
+// 64 matrices of N_aux 1100 2.2 and 1.4 ms. With many matrices the planes' traffic (8 floats per complex value) bounds it.
+__global__ void __launch_bounds__(ROWS_THREADS)
+    ldlt_rows_kernel(float2* __restrict__ mats, int n, int nrow, long long ldm, long long stride, int k0, int koff,
+                     const int* __restrict__ active, const float2* __restrict__ xd, float* __restrict__ ap,
+                     float* __restrict__ bp) {
   const int f = blockIdx.y;
   if (active && !active[f]) return;
-  const float2* A = mats + f * stride;
-  const int kb = min(PW, n - k0), R0 = k0 + kb;
-  const size_t a_plane = (size_t)gridDim.y * nrow * KW, b_plane = (size_t)gridDim.y * n * KW;
-  if ((int)blockIdx.x < nA) {
-    const int i = R0 + 4 * blockIdx.x + (threadIdx.x >> 6), l = threadIdx.x & 63;
-    if (i >= nrow) return;
-    const float2 v = l < kb ? A[(long long)i * ldm + k0 + l] : make_float2(0.f, 0.f);
-    const size_t o = ((size_t)f * nrow + i) * KW + koff + l;
-    const float rh = tf32_rn(v.x), ih = tf32_rn(v.y);
-    ap[o] = rh;
-    ap[a_plane + o] = ih;
-    ap[2 * a_plane + o] = tf32_rn(v.x - rh);
-    ap[3 * a_plane + o] = tf32_rn(v.y - ih);
-    return;
+  extern __shared__ uint8_t smem_raw[];
+  float2* xg = reinterpret_cast<float2*>(smem_raw);                        // [64][64], then dinv [64]
+  float2(*ach)[LDP] = reinterpret_cast<float2(*)[LDP]>(xg + XD);           // [64][65]
+  float2* A = mats + f * stride;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int kb = min(PW, n - k0), base = k0 + kb + 64 * blockIdx.x;  // (with columns beyond it, the panel is 64 wide)
+  const float2* src = xd + (size_t)f * XD;
+  for (int e = tid; e < XD / 2; e += ROWS_THREADS) cp_async16(xg + 2 * e, src + 2 * e, true);
+  for (int e = tid; e < 64 * PW; e += ROWS_THREADS) {
+    const int rr = e >> 6, l = e & 63, i = base + rr;
+    if (i < nrow && l < kb) cp_async_elem<8>(&ach[rr][l], A + (long long)i * ldm + k0 + l);
   }
-  __shared__ float2 tile[PW][33];
-  const int j0 = R0 + 32 * (blockIdx.x - nA);
-  for (int e = threadIdx.x; e < PW * 32; e += 256) {
-    const int l = e >> 5, jj = e & 31, j = j0 + jj;
-    tile[l][jj] = (l < kb && j < n) ? A[(long long)(k0 + l) * ldm + j] : make_float2(0.f, 0.f);
-  }
+  cp_commit();
+  cp_wait<0>();
   __syncthreads();
-  for (int e = threadIdx.x; e < PW * 32; e += 256) {
-    const int jj = e >> 6, l = e & 63, j = j0 + jj;
-    if (j >= n) continue;
-    const float2 v = tile[l][jj];
-    const size_t o = ((size_t)f * n + j) * KW + koff + l;
-    const float rh = tf32_rn(v.x), ih = tf32_rn(v.y);
-    bp[o] = rh;
-    bp[b_plane + o] = ih;
-    bp[2 * b_plane + o] = tf32_rn(v.x - rh);
-    bp[3 * b_plane + o] = tf32_rn(v.y - ih);
+  const float2* dinv = xg + PW * PW;
+  const int r = 32 * (warp >> 1) + lane, i = base + r;
+  if (base + 32 * (warp >> 1) >= nrow) return;  // warp-uniform
+  const size_t a_plane = (size_t)gridDim.y * nrow * KW, b_plane = (size_t)gridDim.y * n * KW;
+  const float2* arow = ach[r];
+#pragma unroll 1
+  for (int pass = 0; pass < 4; ++pass) {  // 8 columns each: 16 float2 accumulators stay in registers
+    const int g = (warp & 1) ? 1 + (pass >> 1) : 3 * (pass >> 1);
+    const int c0 = 16 * g + 8 * (pass & 1), lmax = min(c0 + 8, kb);  // X_cl = 0 for l > c
+    if (c0 >= kb) continue;
+    float2 pr[8], pi[8];  // pr[c] = sum a.re (X re, X im), pi[c] = sum a.im (X re, X im)
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+      pr[c] = make_float2(0.f, 0.f);
+      pi[c] = make_float2(0.f, 0.f);
+    }
+#pragma unroll 4
+    for (int l = 0; l < lmax; ++l) {
+      const float2 a = arow[l];
+      const float2 ar = make_float2(a.x, a.x), ai = make_float2(a.y, a.y);
+      const float4* xp = reinterpret_cast<const float4*>(xg + l * PW + c0);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const float4 x = xp[q];
+        const float2 x0 = make_float2(x.x, x.y), x1 = make_float2(x.z, x.w);
+        pr[2 * q] = __ffma2_rn(ar, x0, pr[2 * q]);
+        pi[2 * q] = __ffma2_rn(ai, x0, pi[2 * q]);
+        pr[2 * q + 1] = __ffma2_rn(ar, x1, pr[2 * q + 1]);
+        pi[2 * q + 1] = __ffma2_rn(ai, x1, pi[2 * q + 1]);
+      }
+    }
+    if (i >= nrow) continue;
+    float2 w[8];
+#pragma unroll
+    for (int c = 0; c < 8; ++c) w[c] = make_float2(pr[c].x - pi[c].y, pr[c].y + pi[c].x);
+    float2* rowp = A + (long long)i * ldm + k0 + c0;
+    if (c0 + 8 <= kb) {
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        *reinterpret_cast<float4*>(rowp + 2 * q) = make_float4(w[2 * q].x, w[2 * q].y, w[2 * q + 1].x, w[2 * q + 1].y);
+    } else {
+#pragma unroll
+      for (int c = 0; c < 8; ++c)
+        if (c0 + c < kb) rowp[c] = w[c];
+    }
+    if (!ap) continue;  // the last panel: no trailing matrix
+    store_planes(ap + ((size_t)f * nrow + i) * KW + koff + c0, a_plane, w);
+    if (i < n) {
+#pragma unroll
+      for (int c = 0; c < 8; ++c) w[c] = cmul_rn(w[c], dinv[c0 + c]);
+      store_planes(bp + ((size_t)f * n + i) * KW + koff + c0, b_plane, w);
+    }
   }
 }
 
@@ -1023,7 +1283,9 @@ int launch_ldlt_tc(void* mats, int n, int nrow, long long ldm, long long stride,
   return cudaPeekAtLastError() == cudaSuccess ? 1 : -1;
 }
 
-size_t ldlt_split_bytes(int n, int nrow, int F) { return (size_t)16 * F * KW * ((size_t)nrow + n) + 1024; }
+size_t ldlt_split_bytes(int n, int nrow, int F) {
+  return (size_t)16 * F * KW * ((size_t)nrow + n) + (size_t)F * XD * sizeof(float2) + 1024;
+}
 
 // Returns the launches, -1 on a launch error or bad layout, -2 if unsupported.
 int launch_ldlt_split(void* mats, int n, int nrow, long long ldm, long long stride, int F, const int* active,
@@ -1033,13 +1295,15 @@ int launch_ldlt_split(void* mats, int n, int nrow, long long ldm, long long stri
   if (ldlt_split_bytes(n, nrow, F) > work_bytes || (reinterpret_cast<uintptr_t>(work) & 15)) return -2;
   static bool attr = false;
   if (!attr) {
-    if (cudaFuncSetAttribute(ldlt_panel_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, PANEL_SMEM) != cudaSuccess ||
+    if (cudaFuncSetAttribute(ldlt_diag_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, DIAG_SMEM) != cudaSuccess ||
+        cudaFuncSetAttribute(ldlt_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, ROWS_SMEM) != cudaSuccess ||
         cudaFuncSetAttribute(ldlt_update_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, UP_SMEM) != cudaSuccess)
       return -1;
     attr = true;
   }
   float* ap = static_cast<float*>(work);
   float* bp = ap + (size_t)4 * F * nrow * KW;
+  float2* xd = reinterpret_cast<float2*>(bp + (size_t)4 * F * n * KW);
   UpParams p;
   std::memset(static_cast<void*>(&p), 0, sizeof(p));
   for (int q = 0; q < 4; ++q) {
@@ -1066,14 +1330,14 @@ int launch_ldlt_split(void* mats, int n, int nrow, long long ldm, long long stri
   p.wait_ns = wait_ns;
   float2* A = reinterpret_cast<float2*>(mats);
   int launches = 0;
-  auto panel = [&](int k0) {
-    ldlt_panel_kernel<<<F, NT_PANEL, PANEL_SMEM, s>>>(A, n, nrow, ldm, stride, k0, active, status);
-    ++launches;
-  };
-  auto planes = [&](int k0, int koff) {
+  // panel k0; its planes (unless it is the last one) at K column koff
+  auto panel = [&](int k0, int koff) {
     const int R0 = k0 + std::min(PW, n - k0);
-    const int nA = (nrow - R0 + 3) / 4, nB = (n - R0 + 31) / 32;
-    ldlt_planes_kernel<<<dim3(nA + nB, F), 256, 0, s>>>(A, n, nrow, ldm, stride, k0, koff, nA, active, ap, bp);
+    ldlt_diag_kernel<<<F, DIAG_THREADS, DIAG_SMEM, s>>>(A, n, ldm, stride, k0, active, xd, status);
+    ++launches;
+    if (R0 >= nrow) return;
+    ldlt_rows_kernel<<<dim3((nrow - R0 + 63) / 64, F), ROWS_THREADS, ROWS_SMEM, s>>>(
+        A, n, nrow, ldm, stride, k0, koff, active, xd, R0 < n ? ap : nullptr, R0 < n ? bp : nullptr);
     ++launches;
   };
   auto update = [&](int R0, int nkc, bool one_col) {
@@ -1094,15 +1358,13 @@ int launch_ldlt_split(void* mats, int n, int nrow, long long ldm, long long stri
   for (int k0 = 0; k0 < n;) {
     // panel p at k0, with the planes of its W columns and L rows in K columns 0..63
     const int R0 = k0 + std::min(PW, n - k0);
-    panel(k0);
+    panel(k0, 0);
     if (R0 >= n) break;
-    planes(k0, 0);
     // lookahead: panel p's update of panel p + 1's columns only, then panel p + 1
     update(R0, PW / KH, true);
-    panel(R0);
+    panel(R0, PW);
     const int R1 = R0 + std::min(PW, n - R0);
     if (R1 < n) {
-      planes(R0, PW);
       update(R1, KW / KH, false);  // both panels: K = 128
     }
     if (cudaPeekAtLastError() != cudaSuccess) return -1;
