@@ -20,6 +20,8 @@
 //   * the trailing lower triangle is updated with the rank-64 product W_panel L_panel^T, in
 //     64 x 64 tiles (4 x 4 per thread); both operands are staged through shared memory by
 //     cp.async in 32-deep chunks, double-buffered across chunks and tiles.
+#include <cooperative_groups.h>
+
 #include <algorithm>
 
 #include "gwc_internal.h"
@@ -163,6 +165,230 @@ __global__ void __launch_bounds__(256) ldlt_solve_kernel(const S* __restrict__ m
   }
 }
 
+// The same substitution for few right-hand sides (r <= kFewRhs, the residue and screening calls): u and w exactly as above, with
+// the sums over l in the same order. The kernel above keeps one CTA per matrix on n/64 serial panels and multiplies 64
+// columns whatever r is, so at r = 6 .. 12 it waits on latency: 9.6 ms for 8 matrices of N_aux 2450. Here a cluster of C CTAs
+// holds a matrix's rows (64-row blocks round robin, their running sums in shared memory) and goes right-looking:
+//   solve   the owner of panel k takes its 64 x 64 diagonal block, a warp per right-hand side and two rows per lane (one
+//           exchange per row, no barrier), and puts u into the shared memory of all C CTAs;
+//   update  every CTA subtracts W[rows][panel] u from the rows it owns, W read once through L1.
+// Measured: 8 complex FP32 matrices of N_aux 2450, r = 12, 9.65 -> 0.84 ms; 64 of 1100, r = 6, 2.43 -> 0.29 ms; 8 complex
+// FP64 ones of 1100, 45 -> 2.3 ms. The chain of the n/64 panels bounds it (about 20 us each: 64 exchanges and the cluster
+// barrier). Beyond kFewRhs right-hand sides (the W table, CD-WAC) the kernel above fills the chip.
+constexpr int kFewRhs = 32;
+constexpr int kFewSmem = 200 * 1024;
+constexpr int FQ = 4;  // right-hand sides per thread of the update
+
+__device__ __forceinline__ float shfl_s(float v, int l) { return __shfl_sync(0xffffffffu, v, l); }
+__device__ __forceinline__ double shfl_s(double v, int l) { return __shfl_sync(0xffffffffu, v, l); }
+__device__ __forceinline__ float2 shfl_s(float2 v, int l) { return make_float2(shfl_s(v.x, l), shfl_s(v.y, l)); }
+__device__ __forceinline__ double2 shfl_s(double2 v, int l) { return make_double2(shfl_s(v.x, l), shfl_s(v.y, l)); }
+
+// products and reciprocals with the roundings of the kernel above written out for complex FP32 (the contractions there are the
+// compiler's; here they decide whether the two agree bit by bit)
+template <typename S> __device__ __forceinline__ S fmul(S a, S b) { return smul(a, b); }
+template <> __device__ __forceinline__ float2 fmul<float2>(float2 a, float2 b) {
+  return make_float2(__fmaf_rn(a.x, b.x, -__fmul_rn(a.y, b.y)), __fmaf_rn(a.y, b.x, __fmul_rn(a.x, b.y)));
+}
+template <typename S> __device__ __forceinline__ S finv(S a) { return sinv(a); }
+template <> __device__ __forceinline__ float2 finv<float2>(float2 a) {
+  const float d = __fmaf_rn(a.x, a.x, __fmul_rn(a.y, a.y));
+  return make_float2(__fdiv_rn(a.x, d), __fdiv_rn(-a.y, d));
+}
+
+// elements of S: diagonal block, d, two u buffers, the sums of `blocks` row blocks; then C * r partial results (2 doubles each)
+inline size_t few_elems(int blocks, int rp) { return (size_t)SB * (SB + 1) + SB + 2 * (size_t)SB * rp + (size_t)blocks * SB * rp; }
+
+template <typename S, int QW>  // QW right-hand sides per warp: r <= 8 QW
+__global__ void __launch_bounds__(256) ldlt_solve_few_kernel(const S* __restrict__ mats, int n, long long ldm, long long stride,
+                                                              const S* __restrict__ rhs, int r, long long ldr,
+                                                              long long rhs_stride, const double* __restrict__ bnorm2,
+                                                              double* __restrict__ w, long long w_stride,
+                                                              const int* __restrict__ active) {
+  constexpr int PER = 16 / (int)sizeof(S);
+  namespace cg = cooperative_groups;
+  cg::cluster_group cl = cg::this_cluster();
+  const int C = (int)cl.num_blocks(), rank = (int)cl.block_rank(), f = blockIdx.x / C;
+  if (active && !active[f]) return;  // the whole cluster
+  const S* L = mats + f * stride;
+  const S* Y = rhs + f * rhs_stride;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int np = (n + SB - 1) / SB, cnt = rank < np ? (np - rank + C - 1) / C : 0;  // panels; row blocks owned
+  const int groups = (r + FQ - 1) / FQ, rp = groups * FQ;
+
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  S* us = reinterpret_cast<S*>(smem_raw);            // [2][SB][rp]
+  S* acc = us + 2 * SB * rp;                         // [cnt * SB][rp]
+  S* wd = acc + (size_t)((np + C - 1) / C) * SB * rp;  // [SB][SB + 1]
+  S* dv = wd + SB * (SB + 1);                        // [SB]
+  double* part = reinterpret_cast<double*>(dv + SB);  // [C][r][2] (on rank 0)
+
+  for (int e = tid; e < cnt * SB * rp; e += 256) acc[e] = szero<S>();
+  auto load_diag = [&](int k) {
+    const int k0 = k * SB, kb = min(SB, n - k0);
+    for (int e = tid; e < SB * SB; e += 256) {
+      const int i = e / SB, l = e % SB;
+      if (i < kb && l < i) cp_async_elem<(int)sizeof(S)>(wd + i * (SB + 1) + l, L + (long long)(k0 + i) * ldm + k0 + l);
+    }
+    if (tid < kb) cp_async_elem<(int)sizeof(S)>(dv + tid, L + (long long)(k0 + tid) * ldm + k0 + tid);
+    cp_commit();
+  };
+  double wr[QW], wi[QW];  // sum u_i^2 d_i over this CTA's panels (every lane its rows)
+#pragma unroll
+  for (int t = 0; t < QW; ++t) wr[t] = wi[t] = 0.0;
+  if (rank == 0) load_diag(0);
+  cl.sync();  // every CTA of the cluster runs before u goes into its shared memory
+  for (int k = 0; k < np; ++k) {
+    const int k0 = k * SB, kb = min(SB, n - k0);
+    S* u_k = us + (k & 1) * SB * rp;
+    if (k % C == rank) {
+      cp_wait<0>();
+      __syncthreads();
+      // a warp's right-hand sides warp + 8 t; lane: rows lane and lane + 32
+      const S* ak = acc + (size_t)(k / C) * SB * rp;
+      S v[QW][2], p[QW][2][4], inv[2], d[2];
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int i = lane + 32 * h;
+        d[h] = i < kb ? dv[i] : sfrom<S>(1.0, 0.0);
+        inv[h] = finv(d[h]);
+#pragma unroll
+        for (int t = 0; t < QW; ++t) {
+          const int q = warp + 8 * t;
+          v[t][h] = (i < kb && q < r) ? sadd(Y[(long long)q * ldr + k0 + i], ak[i * rp + q]) : szero<S>();
+#pragma unroll
+          for (int m = 0; m < 4; ++m) p[t][h][m] = szero<S>();
+        }
+      }
+      if (warp < r) {
+#pragma unroll
+        for (int hl = 0; hl < 2; ++hl) {  // rows l of the first, then of the second half
+#pragma unroll 1
+          for (int l4 = 0; l4 < 32; l4 += 4) {
+#pragma unroll
+            for (int m = 0; m < 4; ++m) {
+              const int l = 32 * hl + l4 + m;
+              const S w0 = wd[lane * (SB + 1) + l], w1 = wd[(lane + 32) * (SB + 1) + l];
+#pragma unroll
+              for (int t = 0; t < QW; ++t) {
+                const S* ph = p[t][hl];
+                const S own = fmul(inv[hl], ssub(v[t][hl], sadd(sadd(ph[0], ph[1]), sadd(ph[2], ph[3]))));
+                const S u = shfl_s(own, l4 + m);
+                if (lane == l4 + m) v[t][hl] = own;  // (u_l; the row takes no further updates)
+                if (hl == 0) p[t][0][m] = sadd(p[t][0][m], fmul(w0, u));
+                p[t][1][m] = sadd(p[t][1][m], fmul(w1, u));
+              }
+            }
+          }
+        }
+      }
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int i = lane + 32 * h;
+#pragma unroll
+        for (int t = 0; t < QW; ++t) {
+          const int q = warp + 8 * t;
+          if (i >= kb || q >= r) continue;
+          const S u = v[t][h], x = fmul(d[h], fmul(u, u));
+          wr[t] += sre(x);
+          wi[t] += sim(x);
+          u_k[i * rp + q] = u;
+        }
+      }
+      __syncthreads();
+      for (int o = 1; o < C; ++o) {
+        S* there = cl.map_shared_rank(u_k, (rank + o) % C);
+        for (int e = tid; e < SB * rp; e += 256) there[e] = u_k[e];
+      }
+    }
+    cl.sync();
+    if (k + 1 == np) break;
+    if ((k + 1) % C == rank) load_diag(k + 1);  // (its previous block here was solved before the barrier)
+    const int m0 = k < rank ? 0 : (k - rank) / C + 1;  // first owned block below panel k
+    if (tid < groups * (256 / groups)) {
+      const int q0 = FQ * (tid % groups);
+      for (int row = m0 * SB + tid / groups; row < cnt * SB; row += 256 / groups) {
+        const int gi = (rank + (row / SB) * C) * SB + row % SB;
+        if (gi >= n) break;
+        const S* wrow = L + (long long)gi * ldm + k0;
+        S* ar = acc + (size_t)row * rp + q0;
+        S a[FQ];
+#pragma unroll
+        for (int j = 0; j < FQ; ++j) a[j] = ar[j];
+#pragma unroll 1
+        for (int l0 = 0; l0 < SB; l0 += 4 * PER) {
+          float4 x[4];
+#pragma unroll
+          for (int c = 0; c < 4; ++c) x[c] = __ldg(reinterpret_cast<const float4*>(wrow + l0 + c * PER));
+#pragma unroll
+          for (int c = 0; c < 4; ++c) {
+            const S* xs = reinterpret_cast<const S*>(&x[c]);
+#pragma unroll
+            for (int e = 0; e < PER; ++e) {
+              const S* ul = u_k + (l0 + c * PER + e) * rp + q0;
+#pragma unroll
+              for (int j = 0; j < FQ; ++j) a[j] = sfnms(xs[e], ul[j], a[j]);
+            }
+          }
+        }
+#pragma unroll
+        for (int j = 0; j < FQ; ++j) ar[j] = a[j];
+      }
+    }
+  }
+  double* there = cl.map_shared_rank(part, 0);
+#pragma unroll
+  for (int t = 0; t < QW; ++t) {
+    const int q = warp + 8 * t;
+    for (int o = 16; o > 0; o >>= 1) {
+      wr[t] += __shfl_xor_sync(0xffffffffu, wr[t], o);
+      wi[t] += __shfl_xor_sync(0xffffffffu, wi[t], o);
+    }
+    if (lane == 0 && q < r) {
+      there[(rank * r + q) * 2] = wr[t];
+      there[(rank * r + q) * 2 + 1] = wi[t];
+    }
+  }
+  cl.sync();
+  if (rank == 0 && tid < r) {
+    double a = 0.0, b = 0.0;
+    for (int c = 0; c < C; ++c) {
+      a += part[(c * r + tid) * 2];
+      b += part[(c * r + tid) * 2 + 1];
+    }
+    double* o = w + f * w_stride + (long long)tid * 2;
+    o[0] = a - bnorm2[(long long)f * r + tid];
+    o[1] = b;
+  }
+}
+
+template <typename S, int QW>
+int run_solve_few(const S* mats, int n, long long ldm, long long stride, const S* rhs, int r, long long ldr,
+                  long long rhs_stride, const double* bnorm2, int F, double* w, long long w_stride, const int* active, int C,
+                  size_t sm, cudaStream_t s) {
+  static bool attr = false;
+  if (!attr) {
+    if (cudaFuncSetAttribute(ldlt_solve_few_kernel<S, QW>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFewSmem) != cudaSuccess)
+      return -1;
+    attr = true;
+  }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(F * C);
+  cfg.blockDim = dim3(256);
+  cfg.dynamicSmemBytes = sm;
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = C;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, ldlt_solve_few_kernel<S, QW>, mats, n, ldm, stride, rhs, r, ldr, rhs_stride, bnorm2, w, w_stride,
+                            active) == cudaSuccess
+             ? 1
+             : -1;
+}
+
 template <typename S>
 size_t solve_smem() {
   return SolveSmem<S>::bytes();
@@ -184,6 +410,17 @@ int run_ldlt(S* mats, int n, int nrow, long long ldm, long long stride, int F, c
 template <typename S>
 int run_solve(const S* mats, int n, long long ldm, long long stride, S* rhs, int r, long long ldr, long long rhs_stride,
               const double* bnorm2, int F, double* w, long long w_stride, const int* active, cudaStream_t s) {
+  if (r <= kFewRhs && ldm % 4 == 0 && stride % 4 == 0 && (reinterpret_cast<uintptr_t>(mats) & 15) == 0) {  // 16-byte loads
+    // the smallest cluster that gives every SM a CTA (F C >= 148 .. 160 on these parts), more where the sums need the room
+    const int np = (n + SB - 1) / SB, rp = (r + FQ - 1) / FQ * FQ;
+    for (int C = 1; C <= 8; C <<= 1) {
+      const size_t few = few_elems((np + C - 1) / C, rp) * sizeof(S) + (size_t)C * r * 16;
+      if (few > (size_t)kFewSmem || (C < 8 && C < np && F * C < 152)) continue;
+      if (r <= 8) return run_solve_few<S, 1>(mats, n, ldm, stride, rhs, r, ldr, rhs_stride, bnorm2, F, w, w_stride, active, C, few, s);
+      if (r <= 16) return run_solve_few<S, 2>(mats, n, ldm, stride, rhs, r, ldr, rhs_stride, bnorm2, F, w, w_stride, active, C, few, s);
+      return run_solve_few<S, 4>(mats, n, ldm, stride, rhs, r, ldr, rhs_stride, bnorm2, F, w, w_stride, active, C, few, s);
+    }
+  }
   static bool attr = false;
   const size_t sm = solve_smem<S>();
   if (!attr) {
