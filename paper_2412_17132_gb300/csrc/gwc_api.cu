@@ -22,6 +22,7 @@ namespace {
 thread_local std::string g_create_error;
 
 const double kPi = 3.14159265358979323846;
+const size_t kScreenKeep = (size_t)64 << 20;
 
 gwc_status fail(gwc_ctx* ctx, gwc_status st, const std::string& msg) {
   if (ctx)
@@ -438,10 +439,10 @@ gwc_status enqueue_wim_tail(gwc_ctx* ctx, int k0, int nb, cudaStream_t st) {
     const size_t ebytes = mat_elem_bytes(rk);
     for (int u0 = 0; u0 < nb; u0 += ctx->wim_group) {
       const int ng = std::min(ctx->wim_group, nb - u0);
-      for (int u = 0; u < ng; ++u)
-        LAUNCH(launch_rhs_gather(rk, ctx->d_o_core, ctx->n_aux, ctx->d_rowmap, 1, r, ctx->n_aux,
-                                 (char*)ctx->d_rhs_im + (size_t)u * plane * ctx->ldm * ebytes, ctx->ldm, 0,
-                                 ctx->d_bnorm + (size_t)u * plane, st));
+      // every node takes the same rows of o_core; one launch for the group (33 nodes of 340 states,
+      // N_aux 1190: 33 launches 0.49 ms, one 0.39 ms)
+      LAUNCH(launch_rhs_gather(rk, ctx->d_o_core, ctx->n_aux, nullptr, 0, ng, r, ctx->n_aux, ctx->d_rhs_im, ctx->ldm,
+                               (long long)plane * ctx->ldm, ctx->d_bnorm, st));
       cudaEvent_t evs = ev_begin(ctx, st);
       if (tc) {
         // blocked forward substitution on the tensor cores (real parts of the complex factors), straight into
@@ -506,7 +507,7 @@ gwc_status residue_batches_buf(gwc_ctx* ctx, int n_pairs, const double* z_dev, c
       cudaEvent_t ev = ev_begin(ctx, st);
       LAUNCH(launch_factor(ctx, ck, ctx->d_mats, ctx->n_aux, ctx->n_aux, stride, nb, act, st));
       ev_end(ctx, kClsFactor, ev, st);
-      LAUNCH(launch_rhs_gather(ck, ctx->d_o_core, ctx->n_aux, rows, nb, r, ctx->n_aux, rhs, ctx->ldm, rstride, bnorm, st));
+      LAUNCH(launch_rhs_gather(ck, ctx->d_o_core, ctx->n_aux, rows, 0, nb, r, ctx->n_aux, rhs, ctx->ldm, rstride, bnorm, st));
       cudaEvent_t evs = ev_begin(ctx, st);
       LAUNCH(launch_ldlt_solve_w(ck, ctx->d_mats, ctx->n_aux, ctx->ldm, stride, rhs, r, ctx->ldm, rstride, bnorm, nb, wout,
                                  (long long)r * 2, act, st));
@@ -778,13 +779,6 @@ gwc_status gwc_create(gwc_ctx** out, const gwc_system* s, const gwc_options* o, 
   CTRY(dalloc(ctx, &ctx->d_active, ctx->batch));
   CTRY(dalloc(ctx, &ctx->d_bnorm, std::max(wim_rows, (size_t)ctx->batch * s->n_core)));
   CTRY(dalloc(ctx, &ctx->d_wtmp, 2 * std::max(wim_rows, (size_t)ctx->batch * s->n_core)));
-  CTRY(dalloc(ctx, &ctx->d_rowmap, plane));
-  {
-    std::vector<int> ident(plane);
-    for (size_t i = 0; i < plane; ++i) ident[i] = (int)i;
-    if (cudaMemcpy(ctx->d_rowmap, ident.data(), sizeof(int) * plane, cudaMemcpyHostToDevice) != cudaSuccess)
-      return bail(fail(ctx, GWC_ERR_CUDA, "rowmap upload failed"));
-  }
   // QP buffers
   {
     const size_t np = (size_t)s->n_core * s->n_occ;
@@ -850,9 +844,6 @@ gwc_status reshape(gwc_ctx* ctx, const gwc_system* s) {
   const long long wg = std::min<long long>({(long long)(c.rhs_im_bytes / per_node), b, (long long)ctx->opt.n_im + 1,
                                             (long long)(c.bnorm / plane)});
   if (b < 1 || wg < 1) return fail(ctx, GWC_ERR_INVALID_ARG, "system does not fit the context's workspace");
-  std::vector<int> ident(plane);
-  for (size_t i = 0; i < plane; ++i) ident[i] = (int)i;
-  CU(cudaMemcpy(ctx->d_rowmap, ident.data(), sizeof(int) * plane, cudaMemcpyHostToDevice));
   std::vector<int> rows((size_t)s->n_core * s->n_occ);
   for (int cc = 0; cc < s->n_core; ++cc)
     for (int m = 0; m < s->n_occ; ++m) rows[(size_t)cc * s->n_occ + m] = m * s->n_core + cc;
@@ -893,7 +884,7 @@ void gwc_destroy(gwc_ctx* ctx) {
   if (!ctx) return;
   void* ptrs[] = {ctx->d_eps, ctx->d_o_ov, ctx->d_o_core, ctx->d_vxc, ctx->d_delta, ctx->d_core_idx, ctx->d_group,
                   ctx->d_xi, ctx->d_wxi, ctx->d_wim, ctx->d_sx, ctx->d_vxc_eff, ctx->d_o_hi, ctx->d_o_lo, ctx->d_o_f32,
-                  ctx->d_mats, ctx->d_dtab, ctx->d_z, ctx->d_active, ctx->d_rhs, ctx->d_bnorm, ctx->d_rowmap,
+                  ctx->d_mats, ctx->d_dtab, ctx->d_z, ctx->d_active, ctx->d_rhs, ctx->d_bnorm,
                   ctx->d_wtmp, ctx->d_rhs_im, ctx->d_status, ctx->d_pidx, ctx->d_wres, ctx->d_pair_m, ctx->d_pair_w,
                   ctx->d_grid_w, ctx->d_qp, ctx->d_qp_z, ctx->d_qp_active, ctx->d_qp_fac, ctx->d_qp_w,
                   ctx->d_qp_rowmap, ctx->d_all_done, ctx->d_cw_a, ctx->d_cw_b, ctx->d_coef, ctx->d_tw,
@@ -901,7 +892,7 @@ void gwc_destroy(gwc_ctx* ctx) {
                   ctx->d_req_pair_of, ctx->d_req_w, ctx->d_req_im, ctx->d_req_a, ctx->d_req_nu, ctx->d_req_eqp,
                   ctx->d_req_dh, ctx->d_req_it, ctx->d_eps_g, ctx->d_ev_sig, ctx->d_ev_diff, ctx->d_active_builds,
                   ctx->d_ev_pidx, ctx->d_ev_pm, ctx->d_ev_pw, ctx->d_ev_z, ctx->d_ev_rows, ctx->d_ev_wres, ctx->d_ev_w,
-                  ctx->d_qp_mask, ctx->d_wt, ctx->d_lp};
+                  ctx->d_qp_mask, ctx->d_wt, ctx->d_lp, ctx->d_screen};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   for (auto& r : ctx->ev_pending) {
@@ -938,37 +929,35 @@ gwc_status gwc_screen(gwc_ctx* ctx, const double* z, int F, const double* rhs, i
   cudaStream_t st = (cudaStream_t)stream;
   MatKind ck = cplx_kind(ctx);
   const size_t es = mat_elem_bytes(ck);
-  // per-call scratch for the right-hand sides of one frequency chunk
+  // scratch for the right-hand sides of one frequency chunk, kept by the context while it is small: allocating and freeing
+  // it, and uploading a row map, took 0.33 of the 0.59 ms of a call on one small matrix
   int chunk = std::max(1, std::min(ctx->batch, (int)std::max<size_t>(1, ((size_t)1 << 30) / ((size_t)n_rhs * ctx->ldm * es))));
-  void* d_r = nullptr;
-  double* d_bn = nullptr;
-  int* d_rows = nullptr;
-  size_t nrow = (size_t)chunk * n_rhs;
-  if (cudaMalloc(&d_r, nrow * ctx->ldm * es) != cudaSuccess || cudaMalloc((void**)&d_bn, nrow * sizeof(double)) != cudaSuccess ||
-      cudaMalloc((void**)&d_rows, nrow * sizeof(int)) != cudaSuccess) {
-    cudaFree(d_r);
-    cudaFree(d_bn);
-    cudaFree(d_rows);
-    return fail(ctx, GWC_ERR_OOM, "gwc_screen scratch allocation failed");
+  chunk = std::min(chunk, F);
+  const size_t nrow = (size_t)chunk * n_rhs, rhs_bytes = (nrow * ctx->ldm * es + 255) / 256 * 256;
+  const size_t bytes = rhs_bytes + nrow * sizeof(double);
+  void* scratch = ctx->d_screen;
+  if (bytes > ctx->screen_cap) {
+    scratch = nullptr;
+    if (cudaMalloc(&scratch, bytes) != cudaSuccess) return fail(ctx, GWC_ERR_OOM, "gwc_screen scratch allocation failed");
+    if (bytes <= kScreenKeep) {
+      cudaFree(ctx->d_screen);
+      ctx->d_screen = scratch;
+      ctx->screen_cap = bytes;
+    }
   }
-  std::vector<int> rows(nrow);
+  void* d_r = scratch;
+  double* d_bn = reinterpret_cast<double*>(static_cast<char*>(scratch) + rhs_bytes);
   gwc_status res = GWC_OK;
   const long long stride = (long long)ctx->n_aux * ctx->ldm;
   for (int f0 = 0; f0 < F && res == GWC_OK; f0 += chunk) {
     int nb = std::min(chunk, F - f0);
-    for (size_t i = 0; i < (size_t)nb * n_rhs; ++i) rows[i] = (int)((size_t)f0 * n_rhs + i);
-    if (cudaMemcpyAsync(d_rows, rows.data(), sizeof(int) * nb * n_rhs, cudaMemcpyHostToDevice, st) != cudaSuccess ||
-        cudaStreamSynchronize(st) != cudaSuccess) {
-      res = fail(ctx, GWC_ERR_CUDA, "row map upload failed");
-      break;
-    }
     res = run_chi0(ctx, true, nb, z + 2 * (size_t)f0, nullptr, ctx->d_mats, -1.0, 1.0, 0, st);
     if (res != GWC_OK) break;
     cudaEvent_t evf = ev_begin(ctx, st);
     int n1 = launch_factor(ctx, ck, ctx->d_mats, ctx->n_aux, ctx->n_aux, stride, nb, nullptr, st);
     ev_end(ctx, kClsFactor, evf, st);
-    int n2 = launch_rhs_gather(ck, rhs, ctx->n_aux, d_rows, nb, n_rhs, ctx->n_aux, d_r, ctx->ldm,
-                               (long long)n_rhs * ctx->ldm, d_bn, st);
+    int n2 = launch_rhs_gather(ck, rhs + (size_t)f0 * n_rhs * ctx->n_aux, ctx->n_aux, nullptr, n_rhs, nb, n_rhs, ctx->n_aux, d_r,
+                               ctx->ldm, (long long)n_rhs * ctx->ldm, d_bn, st);
     cudaEvent_t evs = ev_begin(ctx, st);
     int n3 = launch_ldlt_solve_w(ck, ctx->d_mats, ctx->n_aux, ctx->ldm, stride, d_r, n_rhs, ctx->ldm,
                                  (long long)n_rhs * ctx->ldm, d_bn, nb, w + (size_t)f0 * n_rhs * 2, (long long)n_rhs * 2,
@@ -980,9 +969,7 @@ gwc_status gwc_screen(gwc_ctx* ctx, const double* z, int F, const double* rhs, i
     ctx->stats.factor_flop += factor_flop(ctx->n_aux, true, nb);
   }
   cudaStreamSynchronize(st);
-  cudaFree(d_r);
-  cudaFree(d_bn);
-  cudaFree(d_rows);
+  if (scratch != ctx->d_screen) cudaFree(scratch);
   if (res != GWC_OK) return res;
   return check_stream_error(ctx);
 }

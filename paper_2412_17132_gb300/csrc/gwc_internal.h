@@ -209,10 +209,10 @@ int launch_ldlt_solve_w(MatKind kind, const void* mats, int n, long long ldm, lo
                         long long ldr, long long rhs_stride, const double* bnorm2, int F, double* w,
                         long long w_stride, const int* active, cudaStream_t s);
 
-// Convert FP64 right-hand sides to the matrix kind: src rows given by an index map.
+// Convert FP64 right-hand sides to the matrix kind: src rows given by an index map, or (row_of null) rows f row_f + q.
 // dst[f][q][p] = src[row(f,q)][p]; bnorm2[f][q] = sum_p src^2 (FP64).
-int launch_rhs_gather(MatKind kind, const double* src, long long src_row_stride, const int* row_of /*[F*r]*/, int F,
-                      int r, int n_aux, void* dst, long long ldr, long long rhs_stride, double* bnorm2,
+int launch_rhs_gather(MatKind kind, const double* src, long long src_row_stride, const int* row_of /*[F*r] or null*/, int row_f,
+                      int F, int r, int n_aux, void* dst, long long ldr, long long rhs_stride, double* bnorm2,
                       cudaStream_t s);
 
 // Residue batch helpers ------------------------------------------------------------------
@@ -352,10 +352,12 @@ struct gwc_ctx {
   void* d_rhs = nullptr;    // residue RHS [batch][n_core][n_aux] widest kind
   size_t rhs_bytes = 0;
   double* d_bnorm = nullptr;  // [max(batch*n_core, rhs_im)]
-  int* d_rowmap = nullptr;    // [batch * n_core]
   double* d_wtmp = nullptr;   // [max(batch*n_core, wim_group*n_states*n_core)][2]
   void* d_rhs_im = nullptr;   // imaginary-axis RHS [wim_group][n_states*n_core][ldm] (widest real kind)
   unsigned* d_status = nullptr;
+  // right-hand sides and norms of a gwc_screen chunk, kept up to kScreenKeep bytes (larger ones live for the call)
+  void* d_screen = nullptr;
+  size_t screen_cap = 0;
 
   // residue grid plan
   int plan_cap = 0;

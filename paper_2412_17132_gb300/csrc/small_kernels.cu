@@ -54,10 +54,10 @@ __global__ void split_o_kernel(const double* __restrict__ o, int n_aux, int n_ov
 
 template <typename S>
 __global__ void rhs_gather_kernel(const double* __restrict__ src, long long src_row_stride, const int* __restrict__ row_of,
-                                  int r, int n_aux, S* __restrict__ dst, long long ldr, long long rhs_stride,
+                                  int row_f, int r, int n_aux, S* __restrict__ dst, long long ldr, long long rhs_stride,
                                   double* __restrict__ bnorm2) {
   int f = blockIdx.y, q = blockIdx.x;
-  int row = row_of[f * r + q];
+  long long row = row_of ? row_of[f * r + q] : (long long)f * row_f + q;
   const double* s = src + (size_t)row * src_row_stride;
   S* d = dst + f * rhs_stride + q * ldr;
   double acc = 0.0;
@@ -145,21 +145,21 @@ int launch_split_o(const double* o_ov, int n_aux, int n_ov, int n_aux_pad, int n
   return cudaPeekAtLastError() == cudaSuccess ? 1 : -1;
 }
 
-int launch_rhs_gather(MatKind kind, const double* src, long long src_row_stride, const int* row_of, int F, int r,
+int launch_rhs_gather(MatKind kind, const double* src, long long src_row_stride, const int* row_of, int row_f, int F, int r,
                       int n_aux, void* dst, long long ldr, long long rhs_stride, double* bnorm2, cudaStream_t s) {
   dim3 g(r, F);
   switch (kind) {
     case MatKind::RealF32:
-      rhs_gather_kernel<float><<<g, 128, 0, s>>>(src, src_row_stride, row_of, r, n_aux, (float*)dst, ldr, rhs_stride, bnorm2);
+      rhs_gather_kernel<float><<<g, 128, 0, s>>>(src, src_row_stride, row_of, row_f, r, n_aux, (float*)dst, ldr, rhs_stride, bnorm2);
       break;
     case MatKind::CplxF32:
-      rhs_gather_kernel<float2><<<g, 128, 0, s>>>(src, src_row_stride, row_of, r, n_aux, (float2*)dst, ldr, rhs_stride, bnorm2);
+      rhs_gather_kernel<float2><<<g, 128, 0, s>>>(src, src_row_stride, row_of, row_f, r, n_aux, (float2*)dst, ldr, rhs_stride, bnorm2);
       break;
     case MatKind::RealF64:
-      rhs_gather_kernel<double><<<g, 128, 0, s>>>(src, src_row_stride, row_of, r, n_aux, (double*)dst, ldr, rhs_stride, bnorm2);
+      rhs_gather_kernel<double><<<g, 128, 0, s>>>(src, src_row_stride, row_of, row_f, r, n_aux, (double*)dst, ldr, rhs_stride, bnorm2);
       break;
     case MatKind::CplxF64:
-      rhs_gather_kernel<double2><<<g, 128, 0, s>>>(src, src_row_stride, row_of, r, n_aux, (double2*)dst, ldr, rhs_stride, bnorm2);
+      rhs_gather_kernel<double2><<<g, 128, 0, s>>>(src, src_row_stride, row_of, row_f, r, n_aux, (double2*)dst, ldr, rhs_stride, bnorm2);
       break;
   }
   return cudaPeekAtLastError() == cudaSuccess ? 1 : -1;
