@@ -51,6 +51,17 @@ struct FactorSmem {
   static constexpr size_t bytes() { return sizeof(S) * (2 * STAGE + CS); }
 };
 
+// acc[b] -= sum_l x[l] y[l][16 b], b < NBK, of one row
+template <typename S, int NBK>
+__device__ __forceinline__ void update_row_block(const S* __restrict__ x, const S* __restrict__ y, int lmax, S (&acc)[4]) {
+#pragma unroll 2
+  for (int l = 0; l < lmax; ++l) {
+    const S xa = x[l];
+#pragma unroll
+    for (int b = 0; b < NBK; ++b) acc[b] = sfnms(xa, y[l * TT + 16 * b], acc[b]);
+  }
+}
+
 // A[i][j] -= sum_{l in [k0, k0+klen)} W[i][l] L[j][l] for rows [r0, n), columns [c0, c1), j <= i
 // (n counts every row, including appended right-hand-side rows; c1 never exceeds the factored
 // columns). W is read from the lower part (row i), L from the upper part (row l, column j).
@@ -151,17 +162,36 @@ __device__ void update_region(S* __restrict__ A, int n, long long ldm, int r0, i
     const int lmax = min(KC, k0 + klen - kc);
     const S* X = buf;
     const S* Y = buf + SM::XS;
+    if constexpr (sizeof(typename ST<S>::R) == 8) {
+      // FP64 (the FP64 pipe is the bound): row block a of the tile takes only the 16-column blocks on or below the diagonal
+      // and inside the matrix, by real branches (predicated-off FP64 instructions still take the pipe)
+      const int ri = r0 + TT * it_comp.tI, cj = c0 + TT * it_comp.tJ;
+      const int nc = min(4, (c1 - cj + 15) / 16);
+#pragma unroll
+      for (int a = 0; a < 4; ++a) {
+        const int nb = ri + 16 * a < n ? min(nc, (ri + 16 * a + 15 - cj) / 16 + 1) : 0;
+        const S* xr = X + (ty + 16 * a) * (KC + SM::PADX);
+        switch (nb) {
+          case 4: update_row_block<S, 4>(xr, Y + tx, lmax, acc[a]); break;
+          case 3: update_row_block<S, 3>(xr, Y + tx, lmax, acc[a]); break;
+          case 2: update_row_block<S, 2>(xr, Y + tx, lmax, acc[a]); break;
+          case 1: update_row_block<S, 1>(xr, Y + tx, lmax, acc[a]); break;
+          default: break;
+        }
+      }
+    } else {
 #pragma unroll 4
-    for (int l = 0; l < lmax; ++l) {
-      S xa[4], yb[4];
+      for (int l = 0; l < lmax; ++l) {
+        S xa[4], yb[4];
 #pragma unroll
-      for (int a = 0; a < 4; ++a) xa[a] = X[(ty + 16 * a) * (KC + SM::PADX) + l];
+        for (int a = 0; a < 4; ++a) xa[a] = X[(ty + 16 * a) * (KC + SM::PADX) + l];
 #pragma unroll
-      for (int b = 0; b < 4; ++b) yb[b] = Y[l * TT + tx + 16 * b];
+        for (int b = 0; b < 4; ++b) yb[b] = Y[l * TT + tx + 16 * b];
 #pragma unroll
-      for (int a = 0; a < 4; ++a)
+        for (int a = 0; a < 4; ++a)
 #pragma unroll
-        for (int b = 0; b < 4; ++b) acc[a][b] = sfnms(xa[a], yb[b], acc[a][b]);
+          for (int b = 0; b < 4; ++b) acc[a][b] = sfnms(xa[a], yb[b], acc[a][b]);
+      }
     }
     if (it_comp.chunk == nk - 1) {
       const int i0 = r0 + TT * it_comp.tI, j0 = c0 + TT * it_comp.tJ;
@@ -243,6 +273,57 @@ __device__ void factor_diag_warp(S (*lkk)[NB + 1], S* dinv, int kb, int& sing) {
   __syncwarp();
 }
 
+__device__ __forceinline__ double bcast(double v, int l) { return __shfl_sync(0xffffffffu, v, l); }
+__device__ __forceinline__ double2 bcast(double2 v, int l) { return make_double2(bcast(v.x, l), bcast(v.y, l)); }
+
+// Columns j .. j + 7 of the block in factor_diag_regs: v[c] = column j + c of the lane's row, CNT columns still in work.
+template <typename S, int CNT>
+__device__ __forceinline__ void factor_diag_cols(S (&v)[NB], S (*lkk)[NB + 1], S* dinv, int j0, int kb, int& sing) {
+  const int i = threadIdx.x & 31;
+#pragma unroll 1
+  for (int j = j0; j < min(kb, j0 + 8); ++j) {
+    S d = bcast(v[0], j);
+    const bool zero = sabs2(d) < 1e-60;
+    if (zero) d = sfrom<S>(1.0, 0.0);
+    const S inv = sinv(d), w = v[0], lij = smul(w, inv);
+    if (i > j) {
+      lkk[j][i] = w;  // (above the diagonal: scratch for the row operations of this step)
+      lkk[i][j] = lij;
+    } else if (i == j) {
+      lkk[j][j] = d;
+      dinv[j] = inv;
+      if (zero) sing = 1;
+    }
+    __syncwarp();
+#pragma unroll
+    for (int c = 1; c < CNT; ++c) v[c - 1] = sfnms(lij, lkk[j][min(j + c, NB - 1)], v[c]);  // (beyond the row: not used)
+  }
+}
+
+// The same factorisation with lane i's row in registers, for FP64: the version above reads and writes every element through
+// shared memory, one after the other (a batch of 608 FP64 matrices, two blocks each: 0.98 ms, in registers 0.58 ms).
+template <typename S>
+__device__ void factor_diag_regs(S (*lkk)[NB + 1], S* dinv, int kb, int& sing) {
+  const int i = threadIdx.x & 31;
+  S v[NB];
+#pragma unroll
+  for (int c = 0; c < NB; ++c) v[c] = lkk[i][c];
+  __syncwarp();
+  factor_diag_cols<S, 32>(v, lkk, dinv, 0, kb, sing);
+  factor_diag_cols<S, 24>(v, lkk, dinv, 8, kb, sing);
+  factor_diag_cols<S, 16>(v, lkk, dinv, 16, kb, sing);
+  factor_diag_cols<S, 8>(v, lkk, dinv, 24, kb, sing);
+  __syncwarp();
+}
+
+template <typename S>
+__device__ __forceinline__ void factor_diag(S (*lkk)[NB + 1], S* dinv, int kb, int& sing) {
+  if constexpr (sizeof(typename ST<S>::R) == 8)
+    factor_diag_regs(lkk, dinv, kb, sing);
+  else
+    factor_diag_warp(lkk, dinv, kb, sing);
+}
+
 // diagonal block at (c0, c0): W = L d below the diagonal, d on it, L^T above it
 template <typename S, int NT>
 __device__ void store_diag(S* __restrict__ A, long long ldm, int c0, int kb, S (*lkk)[NB + 1]) {
@@ -276,14 +357,10 @@ __device__ __forceinline__ void solve_row(S (&w)[NB], S (*lkk)[NB + 1], int kb) 
   }
 }
 
-// Factor the panel [k0, k0 + min(PW, n - k0)) (its columns already hold the Schur complement) as
-// two NB-wide halves, on the first NT threads: the diagonal blocks in shared memory (one warp each),
-// then every row below in one pass by one thread: solve against block 1, apply block 1 to its
-// block-2 columns, solve against block 2, and store W (lower) and L^T (upper). Rows >= n are
-// appended right-hand sides (W only).
-template <typename S, int NT>
-__device__ void factor_panel(S* __restrict__ A, int n, int nrow, long long ldm, int k0, const PanelSmem<S, NT>& ps,
-                             int& sing) {
+// Factor the diagonal of the panel [k0, k0 + min(PW, n - k0)) (its columns already hold the Schur complement)
+// as two NB-wide halves, on NT threads: the diagonal blocks in shared memory (one warp each), W, d and L^T stored.
+template <typename S, int NT, typename PS>
+__device__ void factor_panel_diag(S* __restrict__ A, int n, long long ldm, int k0, const PS& ps, int& sing) {
   const int tid = threadIdx.x;
   const int kb = min(PW, n - k0);
   const int kb1 = min(NB, kb), kb2 = kb - kb1;
@@ -294,7 +371,7 @@ __device__ void factor_panel(S* __restrict__ A, int n, int nrow, long long ldm, 
     ps.lkk1[i][j] = (i < kb1 && j <= i) ? A[(long long)(k0 + i) * ldm + (k0 + j)] : szero<S>();
   }
   grp_sync_n<NT>();
-  if (tid < 32) factor_diag_warp(ps.lkk1, ps.dinv1, kb1, sing);
+  if (tid < 32) factor_diag(ps.lkk1, ps.dinv1, kb1, sing);
   grp_sync_n<NT>();
   store_diag<S, NT>(A, ldm, k0, kb1, ps.lkk1);
   if (kb2 > 0) {
@@ -328,12 +405,23 @@ __device__ void factor_panel(S* __restrict__ A, int n, int nrow, long long ldm, 
       ps.lkk2[r][c] = v;
     }
     grp_sync_n<NT>();
-    if (tid < 32) factor_diag_warp(ps.lkk2, ps.dinv2, kb2, sing);
+    if (tid < 32) factor_diag(ps.lkk2, ps.dinv2, kb2, sing);
     grp_sync_n<NT>();
     store_diag<S, NT>(A, ldm, c2, kb2, ps.lkk2);
   }
-  // every row below the panel
-  for (int i = k0 + kb + tid; i < nrow; i += NT) {
+}
+
+// The panel's rows i0, i0 + step, .. < nrow in one pass by one thread each: solve against block 1, apply block 1 to the
+// row's block-2 columns, solve against block 2, and store W (lower) and L^T (upper). Rows >= n are appended
+// right-hand sides (W only).
+template <typename S, int NT>
+__device__ void factor_panel_rows(S* __restrict__ A, int n, int nrow, long long ldm, int k0, const PanelSmem<S, NT>& ps, int i0,
+                                  int step) {
+  const int tid = threadIdx.x;
+  const int kb = min(PW, n - k0);
+  const int kb1 = min(NB, kb), kb2 = kb - kb1;
+  const int c2 = k0 + NB;
+  for (int i = i0; i < nrow; i += step) {
     S* row = A + (long long)i * ldm + k0;
     // block-2 values of the row into this thread's scratch, in flight while block 1 is solved
     S* as = ps.arow + tid;
@@ -376,6 +464,14 @@ __device__ void factor_panel(S* __restrict__ A, int n, int nrow, long long ldm, 
       }
     }
   }
+}
+
+// The whole panel on the first NT threads of one CTA.
+template <typename S, int NT>
+__device__ void factor_panel(S* __restrict__ A, int n, int nrow, long long ldm, int k0, const PanelSmem<S, NT>& ps,
+                             int& sing) {
+  factor_panel_diag<S, NT>(A, n, ldm, k0, ps, sing);
+  factor_panel_rows<S, NT>(A, n, nrow, ldm, k0, ps, k0 + min(PW, n - k0) + (int)threadIdx.x, NT);
   grp_sync_n<NT>();
 }
 
