@@ -1,0 +1,424 @@
+// FP64 polarizability on the tensor cores, by exact products of 8-bit digits (sm_103a: tcgen05 + TMEM + TMA).
+//
+//   Pi_PQ(z_f) = sum_k O_Pk (D_f(k) O_Qk)      (RI polarizability, Sec. "Self-energy evaluation")
+//
+// FP64 arithmetic runs at 1.2 TFLOP/s on this part and bounded the SIMT form (chi0_simt.cu). Here every row of O and of the
+// scaled operand D O (one FP64 product per element, as in the SIMT form) is written as 63-bit fixed-point numbers under the
+// row's own exponent, X = sum_{k<8} a_k 256^k with digits a_k in [-128, 127], which BF16 holds exactly (splitting into exact
+// products: Ozaki, Ogita, Oishi & Rump, Numer. Algorithms 59, 2012). The digit pairs of one order u = k + l are products
+// of small integers whose sums over up to 1024 terms stay below 2^24, so the FP32 accumulator of the tensor core is
+// exact; the orders 7 .. 14 are kept (36 pairs). What is dropped is below 2^-63 of the product of the row maxima:
+// against an extended-precision sum of the same values the error is 5e-17 .. 1.3e-16 of |Pi| (N_ov 416 and 5859, in
+// either part, z near and far from the poles of D), that of the sequential FP64 sum 4e-16 .. 4e-15.
+//
+//   digits_kernel   row exponents, then the eight BF16 digit planes [digit][row][k] of O (once per loaded system) or of
+//                   D O (per frequency part, in chunks of the workspace): integer arithmetic but for the product;
+//   fixed_gemm_kernel  one 128 x 128 tile of the lower triangle per CTA, order by order: TMA-fed digit tiles, four MMAs
+//                   per digit pair and 64-wide chunk into one of two fresh accumulators; segments of at most 1024 terms
+//                   are added, as integers, to a 64-bit sum in TMEM by the fold warps while the next segment runs; after
+//                   the orders (7, 8, 9), (10, 11, 12) and (13, 14) that sum becomes FP64 and is added to the result.
+//
+// Rows with an infinity or NaN (a frequency on a pole) take the FP64 sum in the epilogue, element by element.
+// Every mbarrier wait is bounded (the context's bound); on expiry the CTA records kStatTimeout, drains its copies and MMAs
+// and frees TMEM.
+// Measured against the SIMT form: 8 frequencies of N_aux 1100, N_ov 5859, 137 -> 7.6 ms (digits 0.6 ms); 3133 frequencies of
+// N_aux 200, N_ov 416, 223 -> 30 ms. The digit tiles' way into shared memory bounds it (32 KB per pair and chunk, about 50
+// bytes per cycle and SM; the MMAs alone would take 0.4 of the time). W from it, against quad precision over 48 frequencies of
+// eight systems: geometric mean 5.2e-16 (8.7e-16 with the SIMT form), largest 1.7e-14 (3.1e-14).
+#include <cuda.h>
+
+#include <algorithm>
+#include <cstring>
+
+#include "gwc_internal.h"
+#include "tc_common.cuh"
+
+namespace gwc {
+
+namespace {
+
+constexpr int ND = 8;                    // digits
+constexpr int FT = 128;                  // tile rows and columns
+constexpr int FK = 64;                   // k per chunk (128-byte rows of BF16)
+constexpr int FTILE = FT * FK * 2;       // 16 KB
+constexpr int FST = 6;                   // ring stages, one digit pair each (A tile, B tile)
+constexpr int FTHREADS = 256;            // warp 0 TMA, 1 MMA, 2 TMEM, 4-7 fold
+constexpr int FSMEM = 1024 + FST * 2 * FTILE + 256;
+constexpr int kTerms = 1024;             // 128 * 128 * 1024 = 2^24
+constexpr int kMaxOv = 200000;           // the 64-bit sums stay below 2^51: k * 8 * 2^14 * (2^16 + 2^8 + 1)
+constexpr int kNotFinite = 0x7ff;
+
+constexpr uint32_t kIdescF = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(FT >> 3) << 17) | ((uint32_t)(FT >> 4) << 24);
+
+__device__ __forceinline__ void mma_digits(uint32_t d, uint64_t a, uint64_t b, uint32_t acc) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d),
+      "l"(a), "l"(b), "r"(kIdescF), "r"(acc));
+}
+
+__device__ __forceinline__ void tmem_ld16_nowait(uint32_t taddr, uint32_t (&r)[16]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr));
+}
+
+__device__ __forceinline__ void tmem_st16_u(uint32_t taddr, const uint32_t (&v)[16]) {
+  asm volatile(
+      "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};" ::"r"(taddr),
+      "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]), "r"(v[8]), "r"(v[9]), "r"(v[10]),
+      "r"(v[11]), "r"(v[12]), "r"(v[13]), "r"(v[14]), "r"(v[15])
+      : "memory");
+}
+
+// Fixed point of x under the row's exponent field e (the largest of the row): X = x 2^(62 + 1022 - e) rounded to nearest,
+// |X| <= 2^62, returned with 128 added to every byte: byte k is a_k + 128.
+__device__ __forceinline__ unsigned long long fixed_of(double x, int e) {
+  const unsigned long long bits = (unsigned long long)__double_as_longlong(x);
+  const int ef = (int)(bits >> 52) & 0x7ff;
+  unsigned long long m = (bits & 0xfffffffffffffull) | (ef ? 0x10000000000000ull : 0ull);
+  const int s = max(ef, 1) - e + 9;
+  if (s >= 0)
+    m <<= s;  // at most 9 (10 in a row of denormals)
+  else
+    m = s < -54 ? 0ull : (m + (1ull << (-s - 1))) >> (-s);
+  if ((long long)bits < 0) m = 0ull - m;
+  return m + 0x8080808080808080ull;
+}
+
+// Row blockIdx.x of part blockIdx.y: part zp = zp0 + y of frequency zp / parts scales O by D (dtab null: O itself). ex[y][row] =
+// exponent field of the row's largest element (kNotFinite: some element is not finite); dig[y][digit][row][k].
+__global__ void __launch_bounds__(256) digits_kernel(const double* __restrict__ o, int n_aux, int n_ov, int n_ov_pad, int row0,
+                                                      int rows, const double* __restrict__ dtab, int ld_dtab, int parts, int zp0,
+                                                      const int* __restrict__ active, __nv_bfloat16* __restrict__ dig,
+                                                      int* __restrict__ ex) {
+  const int r = blockIdx.x, P = row0 + r, f = (zp0 + (int)blockIdx.y) / parts, part = (zp0 + (int)blockIdx.y) % parts;
+  if (active && !active[f]) return;
+  const int tid = threadIdx.x;
+  const double* d = dtab ? dtab + ((size_t)f * 2 + part) * ld_dtab : nullptr;
+  const double* row = o + (size_t)P * n_ov;
+  auto value = [&](int k) { return d ? row[k] * d[k] : row[k]; };
+  int e = 0;
+  if (P < n_aux)
+    for (int k = tid; k < n_ov; k += 256) e = max(e, (__double2hiint(value(k)) >> 20) & 0x7ff);
+  __shared__ int red[8];
+  e = __reduce_max_sync(0xffffffffu, e);
+  if ((tid & 31) == 0) red[tid >> 5] = e;
+  __syncthreads();
+#pragma unroll
+  for (int w = 0; w < 8; ++w) e = max(e, red[w]);
+  if (tid == 0) ex[(size_t)blockIdx.y * rows + r] = e;
+  uint8_t* out = reinterpret_cast<uint8_t*>(dig) + (((size_t)blockIdx.y * ND) * rows + r) * (size_t)n_ov_pad * 2;
+  const size_t plane = (size_t)rows * n_ov_pad * 2;
+  for (int k0 = 8 * tid; k0 < n_ov_pad; k0 += 8 * 256) {
+    unsigned long long x[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q)
+      x[q] = (P < n_aux && k0 + q < n_ov) ? fixed_of(value(k0 + q), e) : 0x8080808080808080ull;
+#pragma unroll
+    for (int k = 0; k < ND; ++k) {
+      uint32_t w[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        uint32_t u[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {  // digit as FP32: 2^23 + byte, minus 2^23 + 128; its upper half is the BF16
+          const uint32_t half = k < 4 ? (uint32_t)x[2 * q + h] : (uint32_t)(x[2 * q + h] >> 32);
+          u[h] = __float_as_uint(__uint_as_float(0x4b000000u | ((half >> (8 * (k & 3))) & 0xffu)) - 8388736.0f);
+        }
+        w[q] = __byte_perm(u[0], u[1], 0x7632);
+      }
+      *reinterpret_cast<uint4*>(out + k * plane + (size_t)k0 * 2) = make_uint4(w[0], w[1], w[2], w[3]);
+    }
+  }
+}
+
+struct FixedParams {
+  CUtensorMap a, b;      // digits of O [ND * n_aux_pad][n_ov_pad], of D O [zps * ND * b_rows][n_ov_pad]; boxes 64 x 128
+  const int* ea;         // [n_aux_pad]
+  const int* eb;         // [zps][b_rows]
+  const double* o;       // FP64 rows and factors, for rows that are not finite
+  const double* dtab;
+  int n_ov, ld_dtab;
+  int n_aux, n_aux_pad;
+  int b_row0, b_rows;    // the rows of Q in the B digits
+  int n_kc;
+  int n_pb;              // 128-row blocks of P
+  int zp0, parts;
+  double alpha, beta;
+  double* out;           // element (P, Q) of matrix f at out[(f mat_stride + P ldm + Q) parts + part]
+  long long ldm, mat_stride;
+  const int* active;
+  unsigned* status;
+  unsigned long long wait_ns;
+};
+
+// 2^(e - 1032): the unit of a row with exponent field e (the sums carry 2^104)
+__device__ __forceinline__ double row_unit(int e) {
+  return e > 9 && e < kNotFinite ? __hiloint2double((e - 9) << 20, 0) : scalbn(1.0, e - 1032);
+}
+
+// Orders in the sequence of the sums: 7 .. 14, order u of 15 - u digit pairs (k from u - 7), in segments of seg_chunks(u) chunks.
+__device__ __forceinline__ int seg_chunks(int u) { return kTerms / FK / (15 - u); }
+
+__global__ void __launch_bounds__(FTHREADS, 1) fixed_gemm_kernel(const __grid_constant__ FixedParams p) {
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+  uint64_t* full = reinterpret_cast<uint64_t*>(base + FST * 2 * FTILE);
+  uint64_t* empty = full + FST;
+  uint64_t* seg_full = empty + FST;   // [2] fresh accumulator complete
+  uint64_t* seg_free = seg_full + 2;  // [2] folded
+  uint64_t* done = seg_free + 2;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 1);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+
+  const int zp = p.zp0 + blockIdx.y, f = zp / p.parts, part = zp % p.parts;
+  if (p.active && !p.active[f]) return;  // uniform, before any barrier or TMEM use
+  int t = blockIdx.x, iq = p.b_row0 / FT;  // tile t: Q blocks of this launch in order, P blocks iq .. n_pb - 1 of each
+  while (t >= p.n_pb - iq) {
+    t -= p.n_pb - iq;
+    ++iq;
+  }
+  const int P0 = (iq + t) * FT, Q0 = iq * FT;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+
+  if (threadIdx.x == 0) {
+    for (int i = 0; i < FST; ++i) {
+      mbar_init(smem_u32(&full[i]), 1);
+      mbar_init(smem_u32(&empty[i]), 1);
+    }
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(smem_u32(&seg_full[i]), 1);
+      mbar_init(smem_u32(&seg_free[i]), 4);
+    }
+    mbar_init(smem_u32(done), 1);
+    *abort_flag = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 2) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_u32(tmem_slot)));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = *tmem_slot;  // columns: fresh 0, fresh 1, low and high words of the 64-bit sums
+
+  if (warp == 0) {
+    if (lane == 0) {
+      int n = 0;
+      bool ok = true;
+      const int by = (int)blockIdx.y * ND * p.b_rows + (Q0 - p.b_row0);
+      for (int u = 7; u <= 14 && ok; ++u)
+        for (int c0 = 0; c0 < p.n_kc && ok; c0 += seg_chunks(u))
+          for (int kc = c0; kc < min(p.n_kc, c0 + seg_chunks(u)) && ok; ++kc)
+            for (int k = u - 7; k <= 7; ++k, ++n) {
+              const int s = n % FST;
+              ok = mbar_wait(smem_u32(&empty[s]), ((uint32_t)(n / FST) & 1) ^ 1, abort_flag, p.wait_ns);
+              if (!ok) break;
+              mbar_expect_tx(smem_u32(&full[s]), 2 * FTILE);
+              uint8_t* st = base + s * 2 * FTILE;
+              tma_load_2d(smem_u32(st), &p.a, kc * FK, k * p.n_aux_pad + P0, smem_u32(&full[s]));
+              tma_load_2d(smem_u32(st + FTILE), &p.b, kc * FK, by + (u - k) * p.b_rows, smem_u32(&full[s]));
+            }
+      for (int c = n > FST ? n - FST : 0; c < n; ++c) mbar_drain(smem_u32(&full[c % FST]), (uint32_t)(c / FST) & 1);
+    }
+  } else if (warp == 1) {
+    if (lane == 0) {
+      int n = 0, seg = 0;
+      bool ok = true;
+      for (int u = 7; u <= 14 && ok; ++u)
+        for (int c0 = 0; c0 < p.n_kc && ok; c0 += seg_chunks(u), ++seg) {
+          const uint32_t d = tmem + (uint32_t)((seg & 1) * FT);
+          if (seg >= 2) ok = mbar_wait(smem_u32(&seg_free[seg & 1]), (uint32_t)((seg >> 1) - 1) & 1, abort_flag, p.wait_ns);
+          tc_fence_after();
+          uint32_t acc = 0;
+          for (int kc = c0; kc < min(p.n_kc, c0 + seg_chunks(u)) && ok; ++kc)
+            for (int k = u - 7; k <= 7; ++k, ++n) {
+              const int s = n % FST;
+              ok = mbar_wait(smem_u32(&full[s]), (uint32_t)(n / FST) & 1, abort_flag, p.wait_ns);
+              if (!ok) break;
+              tc_fence_after();
+              const uint32_t st = smem_u32(base + s * 2 * FTILE);
+              const uint64_t da = sdesc(st), db = sdesc(st + FTILE);
+#pragma unroll
+              for (int q = 0; q < FK / 16; ++q) {
+                mma_digits(d, da + 2u * q, db + 2u * q, acc);
+                acc = 1;
+              }
+              mma_commit(smem_u32(&empty[s]));
+            }
+          if (ok) mma_commit(smem_u32(&seg_full[seg & 1]));
+        }
+      mma_commit(smem_u32(done));
+    }
+  } else if (warp >= 4) {
+    // ---- fold and epilogue: a TMEM lane (row of P) per thread ---------------------------------------
+    const int q = warp & 3, P = P0 + 32 * q + lane;
+    const uint32_t lb = tmem + ((uint32_t)(32 * q) << 16);
+    const int* eb = p.eb + (size_t)blockIdx.y * p.b_rows + (Q0 - p.b_row0);
+    const int ea = p.ea[P];
+    const double sa = row_unit(ea);
+    double* o = p.out + ((long long)f * p.mat_stride + (long long)P * p.ldm + Q0) * p.parts + part;
+    const int jlim = P < p.n_aux ? min(FT, min(p.n_aux, P + 1) - Q0) : 0;  // columns written: the lower triangle
+    int seg = 0;
+    bool ok = true;
+    for (int u = 7; u <= 14 && ok; ++u) {
+      const int g = (u - 7) / 3, sh = 8 * ((u - 7) % 3);
+      const bool first = sh == 0, last = sh == 16 || u == 14;  // order of its group
+      for (int c0 = 0; c0 < p.n_kc && ok; c0 += seg_chunks(u), ++seg) {
+        const bool start = first && c0 == 0, end = last && c0 + seg_chunks(u) >= p.n_kc;
+        ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&seg_full[seg & 1]), (uint32_t)(seg >> 1) & 1, abort_flag, p.wait_ns));
+        if (!ok) break;
+        tc_fence_after();
+        const uint32_t fr = lb + (uint32_t)((seg & 1) * FT);
+#pragma unroll 1
+        for (int c = 0; c < FT; c += 16) {
+          uint32_t x[16], lo[16], hi[16];
+          tmem_ld16_nowait(fr + c, x);
+          if (!start) {
+            tmem_ld16_nowait(lb + 2 * FT + c, lo);
+            tmem_ld16_nowait(lb + 3 * FT + c, hi);
+          }
+          asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+          long long v[16];
+#pragma unroll
+          for (int j = 0; j < 16; ++j) {
+            const long long old = start ? 0 : (long long)(((unsigned long long)hi[j] << 32) | lo[j]);
+            v[j] = old + ((long long)__float2int_rn(__uint_as_float(x[j])) << sh);
+          }
+          if (!end) {
+#pragma unroll
+            for (int j = 0; j < 16; ++j) {
+              lo[j] = (uint32_t)v[j];
+              hi[j] = (uint32_t)((unsigned long long)v[j] >> 32);
+            }
+            tmem_st16_u(lb + 2 * FT + c, lo);
+            tmem_st16_u(lb + 3 * FT + c, hi);
+          } else {
+            // the group's sum as FP64 (|v| < 2^51: 1.5 2^52 + v is exact), 256^(3 g - 6) of the last group's unit
+            const double w = g == 0 ? 0x1p-48 : g == 1 ? 0x1p-24 : 1.0;
+#pragma unroll
+            for (int j = 0; j < 16; ++j) {
+              if (c + j >= jlim) continue;
+              const double y = __longlong_as_double(0x4338000000000000ll + v[j]) - 0x1.8p52;
+              double* e = o + (long long)(c + j) * p.parts;
+              double r = g == 0 ? y * w : fma(y, w, *e);
+              if (g == 2) {
+                r = (r * sa) * row_unit(eb[c + j]);
+                if (ea == kNotFinite || eb[c + j] == kNotFinite) {
+                  const double* op = p.o + (size_t)P * p.n_ov;
+                  const double* oq = p.o + (size_t)(Q0 + c + j) * p.n_ov;
+                  const double* d = p.dtab + ((size_t)f * 2 + part) * p.ld_dtab;
+                  r = 0.0;
+                  for (int k = 0; k < p.n_ov; ++k) r = fma(op[k], oq[k] * d[k], r);
+                }
+                r = p.alpha * r + (part == 0 && P == Q0 + c + j ? p.beta : 0.0);
+              }
+              *e = r;
+            }
+          }
+        }
+        tmem_wait_st();
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(smem_u32(&seg_free[seg & 1]));
+      }
+    }
+  }
+  // every MMA issued has completed before TMEM is freed
+  if (warp == 2) {
+    if (lane == 0) mbar_drain(smem_u32(done), 0);
+    __syncwarp();
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (threadIdx.x == 0 && *abort_flag) atomicOr(p.status, kStatTimeout);
+  if (warp == 2) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem));
+  }
+}
+
+}  // namespace
+
+size_t chi0_fixed_digits_bytes(int n_aux_pad, int n_ov_pad) { return (size_t)n_aux_pad * n_ov_pad * 2 * ND; }
+
+size_t chi0_fixed_work_bytes(int n_ov_pad, long long rows) {
+  return (size_t)rows * ((size_t)n_ov_pad * 2 * ND + sizeof(int)) + 1024;
+}
+
+bool chi0_fixed_fits(int n_aux, long long n_ov) { return n_aux >= kFixedMinAux && n_ov <= kMaxOv && tc_supported(); }
+
+int launch_chi0_digits(const double* o, int n_aux, int n_ov, int n_aux_pad, int n_ov_pad, void* digits, int* ex,
+                       cudaStream_t s) {
+  digits_kernel<<<dim3(n_aux_pad, 1), 256, 0, s>>>(o, n_aux, n_ov, n_ov_pad, 0, n_aux_pad, nullptr, 0, 1, 0, nullptr,
+                                                   static_cast<__nv_bfloat16*>(digits), ex);
+  return cudaPeekAtLastError() == cudaSuccess ? 1 : -1;
+}
+
+int launch_chi0_fixed(bool complex_out, const double* o, const void* digits, const int* ex, int n_aux, int n_aux_pad, int n_ov,
+                      int n_ov_pad, const double* dtab, int ld_dtab, int F, double alpha, double beta, void* out, long long ldm,
+                      long long mat_stride, const int* active, void* work, size_t work_bytes, unsigned* status,
+                      unsigned long long wait_ns, cudaStream_t s) {
+  if (!tc_supported()) return -2;
+  const int parts = complex_out ? 2 : 1, n_zp = F * parts, n_pb = n_aux_pad / FT;
+  // per row of the B digits: the planes and an exponent
+  const size_t row = (size_t)n_ov_pad * 2 * ND + sizeof(int);
+  const long long rows_fit = (long long)((work_bytes - 1024) / row);
+  if (work_bytes < 1024 || rows_fit < FT || (reinterpret_cast<uintptr_t>(work) & 127) || n_aux_pad % FT || n_ov_pad % FK) return -2;
+  const int b_rows = (int)std::min<long long>(n_aux_pad, rows_fit / FT * FT);  // Q rows per launch
+  const int zps = (int)std::min<long long>(std::min<long long>(n_zp, 65535), std::max<long long>(1, rows_fit / b_rows));
+  static bool attr = false;
+  if (!attr) {
+    if (cudaFuncSetAttribute(fixed_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, FSMEM) != cudaSuccess) return -1;
+    attr = true;
+  }
+  FixedParams p;
+  std::memset(static_cast<void*>(&p), 0, sizeof(p));
+  p.ea = ex;
+  p.o = o;
+  p.dtab = dtab;
+  p.n_ov = n_ov;
+  p.ld_dtab = ld_dtab;
+  p.n_aux = n_aux;
+  p.n_aux_pad = n_aux_pad;
+  p.n_kc = n_ov_pad / FK;
+  p.n_pb = n_pb;
+  p.parts = parts;
+  p.alpha = alpha;
+  p.beta = beta;
+  p.out = static_cast<double*>(out);
+  p.ldm = ldm;
+  p.mat_stride = mat_stride;
+  p.active = active;
+  p.status = status;
+  p.wait_ns = wait_ns;
+  if (!make_map(&p.a, digits, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, ND * n_aux_pad, n_ov_pad, FK, FT)) return -2;
+  int launches = 0;
+  for (int r0 = 0; r0 < n_aux_pad; r0 += b_rows) {
+    const int rows = std::min(b_rows, n_aux_pad - r0);
+    int tiles = 0;
+    for (int iq = r0 / FT; iq < (r0 + rows) / FT; ++iq) tiles += n_pb - iq;
+    for (int z0 = 0; z0 < n_zp; z0 += zps) {
+      const int nz = std::min(zps, n_zp - z0);
+      int* eb = reinterpret_cast<int*>(static_cast<char*>(work) + (size_t)nz * rows * n_ov_pad * 2 * ND);
+      digits_kernel<<<dim3(rows, nz), 256, 0, s>>>(o, n_aux, n_ov, n_ov_pad, r0, rows, dtab, ld_dtab, parts, z0, active,
+                                                   static_cast<__nv_bfloat16*>(work), eb);
+      p.eb = eb;
+      p.b_row0 = r0;
+      p.b_rows = rows;
+      p.zp0 = z0;
+      if (!make_map(&p.b, work, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, nz * ND * rows, n_ov_pad, FK, FT)) return -2;
+      fixed_gemm_kernel<<<dim3(tiles, nz), FTHREADS, FSMEM, s>>>(p);
+      launches += 2;
+      if (cudaPeekAtLastError() != cudaSuccess) return -1;
+    }
+  }
+  return launches;
+}
+
+}  // namespace gwc

@@ -252,6 +252,13 @@ size_t per_matrix_bytes(const gwc_system* s, const Sizes& z) {
   return (size_t)s->n_aux * z.ldm * z.elem_c + (size_t)s->n_core * z.ldm * z.elem_c + 2 * (size_t)z.ld_dtab * 8 + 256;
 }
 
+// Workspace of the FP64 polarizability: the scaled operand's digits of a whole batch, at most 1 GiB, at least one 128-row block.
+// (With 256 MB, launches of 90 tiles left SMs idle: 8 frequencies of N_aux 1100 9.3 ms, with 1 GiB 7.0 ms, with 2 GiB 5.9 ms.)
+size_t fixed_work_bytes(const Sizes& z, int batch) {
+  const size_t all = chi0_fixed_work_bytes(z.n_ov_pad, 2LL * batch * z.n_aux_pad);
+  return std::max(chi0_fixed_work_bytes(z.n_ov_pad, 128), std::min(all, (size_t)1 << 30));
+}
+
 size_t resident_bytes(const gwc_system* s, const gwc_options* o, const Sizes& z) {
   size_t n_ov = (size_t)s->n_occ * (s->n_states - s->n_occ);
   size_t b = 0;
@@ -262,6 +269,8 @@ size_t resident_bytes(const gwc_system* s, const gwc_options* o, const Sizes& z)
   b += (size_t)s->n_states * s->n_core * z.ldm * z.elem_r;          // imaginary-axis RHS
   b += (size_t)s->n_states * s->n_core * (8 + 16 + 4);              // bnorm, w tmp, rowmap
   if (o->prec != GWC_PREC_FP64) b += (size_t)z.n_aux_pad * z.n_ov_pad * (2 + 2 + 4);
+  if (o->prec == GWC_PREC_FP64 && chi0_fixed_fits(s->n_aux, (long long)n_ov))
+    b += chi0_fixed_digits_bytes(z.n_aux_pad, z.n_ov_pad) + fixed_work_bytes(z, o->batch > 0 ? o->batch : 512);
   return b;
 }
 
@@ -309,6 +318,8 @@ gwc_status load_system(gwc_ctx* ctx, const gwc_system* s, cudaStream_t st) {
   if (ctx->opt.prec != GWC_PREC_FP64)
     LAUNCH(launch_split_o(ctx->d_o_ov, ctx->n_aux, ctx->n_ov, ctx->n_aux_pad, ctx->n_ov_pad, ctx->d_o_hi, ctx->d_o_lo,
                           ctx->d_o_f32, st));
+  if (ctx->chi0_fixed)
+    LAUNCH(launch_chi0_digits(ctx->d_o_ov, ctx->n_aux, ctx->n_ov, ctx->n_aux_pad, ctx->n_ov_pad, ctx->d_o_dig, ctx->d_o_ex, st));
   LAUNCH(launch_sigma_x(ctx->d_o_core, ctx->n_occ, ctx->n_core, ctx->n_aux, ctx->d_sx, st));
   ctx->vxc_given = s->vxc != nullptr;
   if (s->vxc)
@@ -328,7 +339,13 @@ gwc_status run_chi0_any(gwc_ctx* ctx, bool complex_z, int F, const double* d_z, 
   LAUNCH(launch_dtable(d_z, F, ctx->d_delta, ctx->n_ov, ctx->ld_dtab, !fp64, ctx->d_dtab, st));
   MatKind kind = complex_z ? cplx_kind(ctx) : real_kind(ctx);
   cudaEvent_t ev = ev_begin(ctx, st);
-  if (prec == GWC_PREC_FP64) {
+  if (prec == GWC_PREC_FP64 && ctx->chi0_fixed && !full) {
+    const int n = launch_chi0_fixed(complex_z, ctx->d_o_ov, ctx->d_o_dig, ctx->d_o_ex, ctx->n_aux, ctx->n_aux_pad, ctx->n_ov,
+                                    ctx->n_ov_pad, (const double*)ctx->d_dtab, ctx->ld_dtab, F, alpha, beta, out, ctx->ldm, stride,
+                                    active, ctx->d_fx, ctx->fx_bytes, ctx->d_status, ctx->wait_ns, st);
+    if (n == -2) return fail(ctx, GWC_ERR_UNSUPPORTED, "FP64 tensor-core chi0 not available for this shape/device");
+    LAUNCH(n);
+  } else if (prec == GWC_PREC_FP64) {
     LAUNCH(launch_chi0_simt(kind, ctx->d_o_ov, ctx->n_ov, ctx->n_aux, ctx->n_ov, ctx->d_dtab, ctx->ld_dtab, F, alpha, beta,
                             out, ctx->ldm, stride, full, active, st));
   } else if (prec == GWC_PREC_FP32) {
@@ -712,6 +729,16 @@ gwc_status gwc_create(gwc_ctx** out, const gwc_system* s, const gwc_options* o, 
     CTRY(dalloc(ctx, &ctx->d_o_lo, np));
     CTRY(dalloc(ctx, &ctx->d_o_f32, np));
   }
+  // (digits of O: 16 bytes per element; a context that cannot have them keeps the SIMT build)
+  if (o->prec == GWC_PREC_FP64 && chi0_fixed_fits(s->n_aux, (long long)n_ov)) {
+    ctx->dig_cap = chi0_fixed_digits_bytes(z.n_aux_pad, z.n_ov_pad);
+    char* p = nullptr;
+    CTRY(dalloc(ctx, &p, ctx->dig_cap));
+    ctx->d_o_dig = p;
+    CTRY(dalloc(ctx, &ctx->d_o_ex, round_up(s->n_aux, 128)));
+    ctx->ex_cap = (size_t)z.n_aux_pad;
+    ctx->chi0_fixed = true;
+  }
   // imaginary grid
   {
     std::vector<double> x, w;
@@ -739,6 +766,12 @@ gwc_status gwc_create(gwc_ctx** out, const gwc_system* s, const gwc_options* o, 
   ctx->batch_cap = ctx->batch;
   ctx->border_max = std::min(s->n_core, 64);
   ctx->mats_bytes = (size_t)ctx->batch * (s->n_aux + ctx->border_max) * z.ldm * z.elem_c;
+  if (ctx->chi0_fixed) {
+    ctx->fx_bytes = fixed_work_bytes(z, ctx->batch);
+    char* p = nullptr;
+    CTRY(dalloc(ctx, &p, ctx->fx_bytes));
+    ctx->d_fx = p;
+  }
   {
     char* p = nullptr;
     CTRY(dalloc(ctx, &p, ctx->mats_bytes));
@@ -861,6 +894,9 @@ gwc_status reshape(gwc_ctx* ctx, const gwc_system* s) {
   ctx->batch = (int)b;
   ctx->border_max = border;
   ctx->wim_group = (int)wg;
+  ctx->chi0_fixed = ctx->d_o_dig && chi0_fixed_fits(s->n_aux, (long long)n_ov) && (size_t)z.n_aux_pad <= ctx->ex_cap &&
+                    chi0_fixed_digits_bytes(z.n_aux_pad, z.n_ov_pad) <= ctx->dig_cap &&
+                    chi0_fixed_work_bytes(z.n_ov_pad, 128) <= ctx->fx_bytes;
   ctx->wtable_tc = ctx->d_wt && wtable_tc_bytes(s->n_aux, (int)plane, (int)wg) <= ctx->wt_bytes;
   ctx->req_n_omega = 0;       // a request plan belongs to the previous system
   ctx->req_n_pairs = 0;
@@ -892,7 +928,7 @@ void gwc_destroy(gwc_ctx* ctx) {
                   ctx->d_req_pair_of, ctx->d_req_w, ctx->d_req_im, ctx->d_req_a, ctx->d_req_nu, ctx->d_req_eqp,
                   ctx->d_req_dh, ctx->d_req_it, ctx->d_eps_g, ctx->d_ev_sig, ctx->d_ev_diff, ctx->d_active_builds,
                   ctx->d_ev_pidx, ctx->d_ev_pm, ctx->d_ev_pw, ctx->d_ev_z, ctx->d_ev_rows, ctx->d_ev_wres, ctx->d_ev_w,
-                  ctx->d_qp_mask, ctx->d_wt, ctx->d_lp, ctx->d_screen};
+                  ctx->d_qp_mask, ctx->d_wt, ctx->d_lp, ctx->d_o_dig, ctx->d_o_ex, ctx->d_fx, ctx->d_screen};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   for (auto& r : ctx->ev_pending) {

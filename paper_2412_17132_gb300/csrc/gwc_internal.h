@@ -122,6 +122,20 @@ int launch_chi0_simt(MatKind kind, const void* o_ov /*double or float [n_aux][ld
                      const void* dtab, int ld_dtab, int F, double alpha, double beta, void* out, long long ldm,
                      long long mat_stride, int full, const int* active, cudaStream_t s);
 
+// FP64 chi0 from exact products of 8-bit digits on the tensor cores: same output contract as launch_chi0_simt for the FP64
+// kinds, lower triangle only. The digits of O (chi0_fixed_digits_bytes bytes) and the exponents of its rows ([n_aux_pad] ints)
+// come from launch_chi0_digits; dtab is the FP64 table; `work` (128-byte aligned) holds the digits of D O in chunks, at least
+// chi0_fixed_work_bytes(n_ov_pad, 128) bytes. Returns the launches, -1 on a launch error, -2 if unsupported.
+constexpr int kFixedMinAux = 64;
+size_t chi0_fixed_digits_bytes(int n_aux_pad, int n_ov_pad);
+size_t chi0_fixed_work_bytes(int n_ov_pad, long long rows);
+bool chi0_fixed_fits(int n_aux, long long n_ov);
+int launch_chi0_digits(const double* o, int n_aux, int n_ov, int n_aux_pad, int n_ov_pad, void* digits, int* ex, cudaStream_t s);
+int launch_chi0_fixed(bool complex_out, const double* o, const void* digits, const int* ex, int n_aux, int n_aux_pad, int n_ov,
+                      int n_ov_pad, const double* dtab, int ld_dtab, int F, double alpha, double beta, void* out, long long ldm,
+                      long long mat_stride, const int* active, void* work, size_t work_bytes, unsigned* status,
+                      unsigned long long wait_ns, cudaStream_t s);
+
 // tcgen05 chi0 (BF16 or split BF16): same output contract as launch_chi0_simt for complex
 // kinds (CplxF32) and real (RealF32). Returns -1 if unavailable.
 int launch_chi0_tc(bool split3, const __nv_bfloat16* o_hi, const __nv_bfloat16* o_lo, const float* o_f32, int ld_pad,
@@ -327,7 +341,11 @@ struct gwc_ctx {
 
   __nv_bfloat16 *d_o_hi = nullptr, *d_o_lo = nullptr;
   float* d_o_f32 = nullptr;
-  float* d_o_f32_unpadded = nullptr;  // not used
+  void* d_o_dig = nullptr;     // FP64 mode: digit planes of O (dig_cap bytes) and the exponents of its rows
+  int* d_o_ex = nullptr;
+  void* d_fx = nullptr;        // FP64 mode: digits of the scaled operand, fx_bytes bytes
+  size_t dig_cap = 0, ex_cap = 0, fx_bytes = 0;
+  bool chi0_fixed = false;     // FP64 polarizabilities from digits on the tensor cores
 
   // workspace
   int batch = 0;            // matrices per batch
