@@ -255,7 +255,8 @@ def load_traffic(kernel, workload, units_per_launch):
 def chi0_kernel_info(n_aux, n_ov):
     """The tensor-core chi0 kernel the library runs (CTA pairs unless GWC_CHI0_KERNEL=single): its name, its
     traffic key and the ratio of executed MMA work (whole 128 x 128 tiles of the padded lower triangle, the
-    pair kernel's 256 x 128 tiles) to the algorithmic N_aux (N_aux + 1) N_ov per part."""
+    pair kernel's 256 x 128 tiles) to the algorithmic N_aux (N_aux + 1) N_ov per part. The pair tiles are counted
+    as 256-row blocks from row 0; with an odd number of 128-row blocks the kernel launches fewer."""
     n_aux_pad = -(-n_aux // 128) * 128
     n_ov_pad = -(-n_ov // 64) * 64
     nqb = n_aux_pad // 128
