@@ -113,8 +113,9 @@ typedef struct {
                             MMAs it issued, frees its tensor memory and records
                             GWC_ERR_TIMEOUT (reported by gwc_sync); the results of that call
                             are undefined, and the context stays usable. 0..60000000          */
-  int chi0_ctas;         /* launch shape of the tensor-core polarizability build: 0 one CTA (or
-                            CTA pair) per (tile, frequency group) item; > 0 at most that many
+  int chi0_ctas;         /* launch shape of the tensor-core polarizability build: 0 chosen by size,
+                            one CTA (or CTA pair) per (tile, frequency group) item or, for
+                            N_ov up to 16384 on CTA pairs, one per SM; > 0 at most that many
                             CTAs, each looping over the items (persistent). gwc_autotune may
                             change it */
   int chi0_tile;         /* tile shape of the tensor-core polarizability build: 0 256 x 128 tiles

@@ -352,10 +352,15 @@ gwc_status run_chi0_any(gwc_ctx* ctx, bool complex_z, int F, const double* d_z, 
     LAUNCH(launch_chi0_simt(kind, ctx->d_o_f32, ctx->n_ov_pad, ctx->n_aux, ctx->n_ov_pad, ctx->d_dtab, ctx->ld_dtab, F,
                             alpha, beta, out, ctx->ldm, stride, full, active, st));
   } else {
+    // Launch shape of the pair kernel where the options leave it open: with few 64-wide chunks per tile a persistent launch, which
+    // keeps TMEM and the barriers and loads the next tile's first chunks under the last one's epilogue, else a CTA pair per
+    // tile. Measured: N_ov 416 x 608 frequencies 233 -> 175 us, 5859 x 64 2149 -> 2074 us, 6099 x 64 2662 -> 2583 us; 25 779
+    // x 8 4896 and 4871 us, 89 571 x 2 12.92 and 12.97 ms.
+    const int ctas = ctx->opt.chi0_ctas > 0 ? ctx->opt.chi0_ctas : ctx->chi0_pair && ctx->n_ov_pad <= 16384 ? ctx->n_sm : 0;
     int n = (ctx->chi0_pair ? launch_chi0_pair : launch_chi0_tc)(
         prec != GWC_PREC_BF16, ctx->d_o_hi, ctx->d_o_lo, ctx->d_o_f32, ctx->n_ov_pad, ctx->n_aux, ctx->n_aux_pad,
         ctx->n_ov_pad, (const float*)ctx->d_dtab, ctx->ld_dtab, F, complex_z, alpha, beta, out, ctx->ldm, stride, active,
-        ctx->d_status, ctx->wait_ns, factor64(prec), st, ctx->opt.chi0_ctas);
+        ctx->d_status, ctx->wait_ns, factor64(prec), st, ctas);
     if (n == -2) return fail(ctx, GWC_ERR_UNSUPPORTED, "tensor-core chi0 not available for this shape/device");
     LAUNCH(n);
     if (full) {
