@@ -94,12 +94,12 @@ __device__ __forceinline__ void split4(const float (&v)[4], float4& hi, float4& 
 // What bounds the block is the chain of its 64 pivots (a reciprocal, two products and an exchange each), not its
 // arithmetic, so the columns go in four blocks of 16:
 //   pivots  one warp factors the 16 x 16 block in registers, two lanes per row;
-//   panel   a thread per row below and a thread per column of X finish the block's columns without any exchange;
+//   panel   four lanes per row below and per column of X finish the block's columns (one exchange per pivot);
 //   update  the next 16 x 16 block by all threads, then the rows below, for a and for X, in 2 x 4 tiles by the other warps
 //           while the first warp takes the next block's pivots.
 // The loops over j keep the current columns in front and shift: unrolled fully they were bound by instruction fetches. With one
-// CTA barrier per pivot and every d_j^-1 W_cj formed again by each thread that uses it a block
-// took 38 us; this takes 27 us (one to 152 matrices).
+// CTA barrier per pivot and every d_j^-1 W_cj formed again by each thread that uses it a block took 38 us; this takes
+// 23 us, about 3.2 us for the 16 pivots of a block and 1.3 us for its panel step.
 constexpr int DB = 16;        // columns per block
 constexpr int LDB = 2 * DB;   // row of the in-block factors (the second half pads the shifted reads)
 constexpr int LDP = PW + 1;   // padded row (conflict-free column access)
@@ -144,16 +144,6 @@ __device__ __forceinline__ float2 shfl2(float2 v, int src) {
   return make_float2(__shfl_sync(0xffffffffu, v.x, src), __shfl_sync(0xffffffffu, v.y, src));
 }
 
-// v[c] -= w m[c] for the columns c = 2 .. 15 beyond an even column 0 (m 16-byte aligned)
-__device__ __forceinline__ void cols_after_even(float2 (&v)[DB], float2 w, const DiagSmem& ds, int m) {
-#pragma unroll
-  for (int c = 2; c < DB; c += 2) {
-    const float4 x = ds.pair(m + c);
-    v[c] = sfnms(w, make_float2(x.x, x.y), v[c]);
-    v[c + 1] = sfnms(w, make_float2(x.z, x.w), v[c + 1]);
-  }
-}
-
 // Pivots of the 16 x 16 block at j0 (its values in ds.dm) by one warp. Lanes i and 16 + i share row i: both carry the current pair
 // of columns (v0, v1), and each the further columns of its parity (f[k] = column 2 + 2k + h of the row, relative to the pair). Of the
 // reciprocal each half forms one part (one division instead of two in the chain), and the next pivot is formed by its own lane.
@@ -174,21 +164,22 @@ __device__ __forceinline__ void diag_pivots(int j0, int w16, const DiagSmem& ds,
   pivot();
   // one column: l = d^-1 w published, the next column `next` updated, its pivot and reciprocal started
   auto column = [&](int j, float2 w, float2& next) {
-    if (lane == j) {
-      ds.dinv(j0 + j) = inv;
-      ds.dpiv(j0 + j) = d;
-      if (zero) *sing = 1;
-    }
-    const float2 l = cmul_rn(inv, w);
+    const float2 l = cmul_rn(inv, w), inv_j = inv, d_j = d;
+    const bool zero_j = zero;
+    const float2 e = sfnms(w, l, next);  // the diagonal entry in lane j + 1
+    d = shfl2(e, j + 1);                 // (after the last column, a value that is not used)
+    next = sfnms(w, shfl2(l, j + 1), next);
     if (i > j && lane < w16) {
       ds.dm(j0 + i, j0 + j) = w;
       ds.wb(j, i) = w;
       ds.lb(j, i) = l;
     }
-    const float2 e = sfnms(w, l, next);  // the diagonal entry in lane j + 1
-    d = shfl2(e, j + 1);                 // (after the last column, a value that is not used)
-    next = sfnms(w, shfl2(l, j + 1), next);
     pivot();
+    if (lane == j) {
+      ds.dinv(j0 + j) = inv_j;
+      ds.dpiv(j0 + j) = d_j;
+      if (zero_j) *sing = 1;
+    }
     __syncwarp();
   };
 #pragma unroll 1
@@ -217,12 +208,60 @@ __device__ __forceinline__ void diag_pivots(int j0, int w16, const DiagSmem& ds,
   }
 }
 
-// v[c] -= w m[c], c >= 1 beyond column 0 of an even pair (first) or c >= 2 beyond column 1 (second)
-__device__ __forceinline__ void panel_step(float2 (&v)[DB], float2 w, const DiagSmem& ds, int m, bool first) {
-  if (first) {
-    v[1] = sfnms(w, ds.at(m + 1), v[1]);
+// The panel step of the block at j0, four lanes per line: the lines t >= j1 are the rows below (their 16 columns of W), the lines t
+// < j1 the columns of X (their 16 rows; zero above the diagonal). Lane s of a line holds its elements s, s + 4, s + 8, s + 12 as v;
+// element j goes from its lane to the others, and each takes it off the elements beyond j. The results are W (ds.dm) or X
+// (ds.xr), and d_j^-1 times them as the update's second operand.
+template <bool COL>
+__device__ __forceinline__ void diag_panel_lines(int j0, int w16, int kb, const DiagSmem& ds) {
+  const int t = threadIdx.x >> 2, s = threadIdx.x & 3, grp = (threadIdx.x & 31) & ~3, line = min(t, kb - 1);
+  float2 v[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) v[q] = COL ? ds.xr(j0 + s + 4 * q, line) : ds.dm(line, j0 + s + 4 * q);
+#pragma unroll 1
+  for (int j4 = 0; j4 < w16; j4 += 4) {
+    float2 own = v[0];  // this lane's element of the four
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const int j = j4 + e, m = (COL ? DiagSmem::WB : DiagSmem::LB) + j * LDB + j4 + s;
+      const float2 x = shfl2(own, grp + e);
+      float2 xs = cmul_rn(ds.dinv(j0 + j), x);
+      if (COL) {  // X_ic -= W_ij (d_j^-1 X_jc), X_jc = 0 above the diagonal
+        const bool on = j0 + j >= t;
+        if (!on) xs = make_float2(0.f, 0.f);
+        const float2 u = sfnms(ds.at(m), xs, own);
+        if (on && s > e) own = u;
+#pragma unroll
+        for (int q = 1; q < 4; ++q) {
+          const float2 y = sfnms(ds.at(m + 4 * q), xs, v[q]);
+          if (on) v[q] = y;
+        }
+      } else {  // a_ic -= W_ij (d_j^-1 W_cj)
+        const float2 u = sfnms(x, ds.at(m), own);
+        if (s > e) own = u;
+#pragma unroll
+        for (int q = 1; q < 4; ++q) v[q] = sfnms(x, ds.at(m + 4 * q), v[q]);
+      }
+      if (s == e && t < kb && j < w16) {
+        if (COL)
+          ds.xr(j0 + j, t) = x;
+        else
+          ds.dm(t, j0 + j) = x;
+        ds.mj(j, t) = xs;
+      }
+    }
+    v[0] = v[1];
+    v[1] = v[2];
+    v[2] = v[3];
   }
-  cols_after_even(v, w, ds, m);
+}
+
+// (8 lines per warp; below the block j1 is a multiple of 16, and with the last block there are no rows: a warp takes one side)
+__device__ __forceinline__ void diag_panel(int j0, int kb, int j1, const DiagSmem& ds) {
+  if ((int)(threadIdx.x >> 2) < j1 || j1 == kb)
+    diag_panel_lines<true>(j0, j1 - j0, kb, ds);
+  else
+    diag_panel_lines<false>(j0, j1 - j0, kb, ds);
 }
 
 // diagonal block [k0, k0 + kb): W and d stored to A (and L^T above the diagonal if `lt`); dinv and xr left in shared memory
@@ -252,54 +291,8 @@ __device__ void factor_diag_block(float2* __restrict__ A, long long ldm, int k0,
   if (tid < 32) diag_pivots(0, min(DB, kb), ds, sing);
   grp_sync_n<NT>();
   for (int j0 = 0; j0 < kb; j0 += DB) {
-    const int w16 = min(DB, kb - j0), j1 = j0 + w16;
-    if (tid < kb - j1) {  // row i below the block: its 16 columns of W, and d^-1 W as the update's second operand
-      const int i = j1 + tid;
-      float2 v[DB];
-#pragma unroll
-      for (int c = 0; c < DB; ++c) v[c] = ds.dm(i, j0 + c);
-#pragma unroll 1
-      for (int j = 0; j < DB; j += 2) {
-        const float2 w0 = v[0];
-        panel_step(v, w0, ds, DiagSmem::LB + j * LDB + j, true);
-        const float2 w1 = v[1];
-        panel_step(v, w1, ds, DiagSmem::LB + (j + 1) * LDB + j, false);
-        ds.dm(i, j0 + j) = w0;
-        ds.dm(i, j0 + j + 1) = w1;
-        ds.mj(j, i) = cmul_rn(ds.dinv(j0 + j), w0);
-        ds.mj(j + 1, i) = cmul_rn(ds.dinv(j0 + j + 1), w1);
-#pragma unroll
-        for (int c = 0; c + 2 < DB; ++c) v[c] = v[c + 2];
-      }
-    } else if (tid >= 64 && tid < 64 + j1) {  // column c of X: its rows in the block (zero above the diagonal)
-      const int c = tid - 64;
-      float2 x[DB];
-#pragma unroll
-      for (int j = 0; j < DB; ++j) x[j] = ds.xr(j0 + j, c);
-#pragma unroll 1
-      for (int j = 0; j < w16; j += 2) {
-#pragma unroll
-        for (int s = 0; s < 2; ++s) {
-          if (j + s >= w16) break;
-          const bool on = j0 + j + s >= c;
-          const float2 xj = x[s], xs = on ? cmul_rn(ds.dinv(j0 + j + s), xj) : make_float2(0.f, 0.f);
-          ds.xr(j0 + j + s, c) = xj;
-          ds.mj(j + s, c) = xs;
-          if (on) {  // x_i -= W_ij (d_j^-1 x_j): the operands in the order of the update below
-            const int m = DiagSmem::WB + (j + s) * LDB + j;
-            if (s == 0) x[1] = sfnms(ds.at(m + 1), xs, x[1]);
-#pragma unroll
-            for (int i = 2; i < DB; i += 2) {
-              const float4 w = ds.pair(m + i);
-              x[i] = sfnms(make_float2(w.x, w.y), xs, x[i]);
-              x[i + 1] = sfnms(make_float2(w.z, w.w), xs, x[i + 1]);
-            }
-          }
-        }
-#pragma unroll
-        for (int i = 0; i + 2 < DB; ++i) x[i] = x[i + 2];
-      }
-    }
+    const int j1 = min(j0 + DB, kb);
+    if (tid < 4 * PW) diag_panel(j0, kb, j1, ds);
     grp_sync_n<NT>();
     const int nr = kb - j1;
     if (nr <= 0) break;  // (below, j1 < kb: the block is full)
@@ -315,10 +308,10 @@ __device__ void factor_diag_block(float2* __restrict__ A, long long ldm, int k0,
     grp_sync_n<NT>();
     if (tid < 32) {
       diag_pivots(j1, min(DB, nr), ds, sing);
-    } else {
+    } else if ((tid >> 5) & 3) {  // (no warp on the first one's scheduler: its chain is the longer of the two)
       // rows below the block: a_ic (c beyond the block) and X_ic (c up to it); a thread's rows are r and r + tr
       const int tr = (nr + 1) >> 1;
-      for (int e = tid - 32; e < tr * (PW / 4); e += NT - 32) {
+      for (int e = tid - 32 - 32 * (tid >> 7); e < tr * (PW / 4); e += NT / 4 * 3) {
         const int r = e % tr, c0 = 4 * (e / tr), i0 = j1 + r, i1 = min(i0 + tr, kb - 1);
         if (c0 > i1 || (c0 >= j1 && i1 < j1 + DB)) continue;  // above the diagonal, or the next 16 x 16 block
         const bool x_side = c0 < j1;  // a tile lies on one side: j1 is a multiple of 4
@@ -995,31 +988,25 @@ __global__ void __launch_bounds__(DIAG_THREADS)
   if (threadIdx.x == 0 && sing) atomicOr(status, kStatSingular);
 }
 
-__device__ __forceinline__ void store_planes(float* __restrict__ o, size_t plane, const float2 (&v)[8]) {
-#pragma unroll
-  for (int q = 0; q < 2; ++q) {
-    float re[4], im[4];
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      re[e] = v[4 * q + e].x;
-      im[e] = v[4 * q + e].y;
-    }
-    float4 rh, rl, ih, il;
-    split4(re, rh, rl);
-    split4(im, ih, il);
-    *reinterpret_cast<float4*>(o + 4 * q) = rh;
-    *reinterpret_cast<float4*>(o + plane + 4 * q) = ih;
-    *reinterpret_cast<float4*>(o + 2 * plane + 4 * q) = rl;
-    *reinterpret_cast<float4*>(o + 3 * plane + 4 * q) = il;
-  }
+// four columns of a row as TF32 hi and lo planes (re hi, im hi, re lo, im lo)
+__device__ __forceinline__ void store_planes(float* __restrict__ o, size_t plane, const float2 (&v)[4]) {
+  const float re[4] = {v[0].x, v[1].x, v[2].x, v[3].x}, im[4] = {v[0].y, v[1].y, v[2].y, v[3].y};
+  float4 rh, rl, ih, il;
+  split4(re, rh, rl);
+  split4(im, ih, il);
+  *reinterpret_cast<float4*>(o) = rh;
+  *reinterpret_cast<float4*>(o + plane) = ih;
+  *reinterpret_cast<float4*>(o + 2 * plane) = rl;
+  *reinterpret_cast<float4*>(o + 3 * plane) = il;
 }
 
 // Rows below panel k0, 64 per CTA (blockIdx.x) of matrix blockIdx.y: W = A X^T, stored to A, and the TF32 hi / lo planes of W
 // (rows i) and of L = W D^-1 (the rows that are columns of the trailing matrix, j < n) that the update reads, K-major at K
 // column koff. Warp w takes the 32-row block w / 2 and the column groups {0, 3} or {1, 2} (equal work: the triangle of X).
 // The rows were the panel CTA's second half, 192 at a time on one SM per matrix (21 us each), and the planes a kernel
-// of their own: 8 matrices of N_aux 2450, panels and planes of a factorisation 7.1 ms, diagonal blocks and rows now 1.8 ms;
-// 64 matrices of N_aux 1100 2.2 and 1.4 ms. With many matrices the planes' traffic (8 floats per complex value) bounds it.
+// of their own: 8 matrices of N_aux 2450, panels and planes of a factorisation 7.1 ms, diagonal blocks and rows now 1.4 ms;
+// 64 matrices of N_aux 1100 2.2 and 0.95 ms. With many matrices the planes' traffic (8 floats per complex value) bounds it: W goes
+// through shared memory so that every plane is written in whole 256-byte row segments (0.94 -> 0.54 ms for the 64).
 __global__ void __launch_bounds__(ROWS_THREADS)
     ldlt_rows_kernel(float2* __restrict__ mats, int n, int nrow, long long ldm, long long stride, int k0, int koff,
                      const int* __restrict__ active, const float2* __restrict__ xd, float* __restrict__ ap,
@@ -1042,15 +1029,13 @@ __global__ void __launch_bounds__(ROWS_THREADS)
   cp_wait<0>();
   __syncthreads();
   const float2* dinv = xg + PW * PW;
-  const int r = 32 * (warp >> 1) + lane, i = base + r;
-  if (base + 32 * (warp >> 1) >= nrow) return;  // warp-uniform
-  const size_t a_plane = (size_t)gridDim.y * nrow * KW, b_plane = (size_t)gridDim.y * n * KW;
+  const int r = 32 * (warp >> 1) + lane;
   const float2* arow = ach[r];
-#pragma unroll 1
-  for (int pass = 0; pass < 4; ++pass) {  // 8 columns each: 16 float2 accumulators stay in registers
+  float2 w[4][8];
+#pragma unroll
+  for (int pass = 0; pass < 4; ++pass) {  // 8 columns each: 16 float2 accumulators
     const int g = (warp & 1) ? 1 + (pass >> 1) : 3 * (pass >> 1);
-    const int c0 = 16 * g + 8 * (pass & 1), lmax = min(c0 + 8, kb);  // X_cl = 0 for l > c
-    if (c0 >= kb) continue;
+    const int c0 = 16 * g + 8 * (pass & 1), lmax = c0 < kb ? min(c0 + 8, kb) : 0;  // X_cl = 0 for l > c
     float2 pr[8], pi[8];  // pr[c] = sum a.re (X re, X im), pi[c] = sum a.im (X re, X im)
 #pragma unroll
     for (int c = 0; c < 8; ++c) {
@@ -1072,26 +1057,39 @@ __global__ void __launch_bounds__(ROWS_THREADS)
         pi[2 * q + 1] = __ffma2_rn(ai, x1, pi[2 * q + 1]);
       }
     }
-    if (i >= nrow) continue;
-    float2 w[8];
 #pragma unroll
-    for (int c = 0; c < 8; ++c) w[c] = make_float2(pr[c].x - pi[c].y, pr[c].y + pi[c].x);
-    float2* rowp = A + (long long)i * ldm + k0 + c0;
-    if (c0 + 8 <= kb) {
+    for (int c = 0; c < 8; ++c) w[pass][c] = make_float2(pr[c].x - pi[c].y, pr[c].y + pi[c].x);
+  }
+  __syncthreads();  // the rows of A have been read: W takes their place, then goes out in whole row segments
 #pragma unroll
-      for (int q = 0; q < 4; ++q)
-        *reinterpret_cast<float4*>(rowp + 2 * q) = make_float4(w[2 * q].x, w[2 * q].y, w[2 * q + 1].x, w[2 * q + 1].y);
+  for (int pass = 0; pass < 4; ++pass) {
+    const int c0 = 16 * ((warp & 1) ? 1 + (pass >> 1) : 3 * (pass >> 1)) + 8 * (pass & 1);
+#pragma unroll
+    for (int c = 0; c < 8; ++c) ach[r][c0 + c] = w[pass][c];
+  }
+  __syncthreads();
+  const size_t a_plane = (size_t)gridDim.y * nrow * KW, b_plane = (size_t)gridDim.y * n * KW;
+  for (int e = tid; e < 64 * 16; e += ROWS_THREADS) {
+    const int rr = e >> 4, c = 4 * (e & 15), i = base + rr;
+    if (i >= nrow || c >= kb) continue;
+    float2 v[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) v[q] = ach[rr][c + q];
+    float2* o = A + (long long)i * ldm + k0 + c;
+    if (c + 4 <= kb) {
+      *reinterpret_cast<float4*>(o) = make_float4(v[0].x, v[0].y, v[1].x, v[1].y);
+      *reinterpret_cast<float4*>(o + 2) = make_float4(v[2].x, v[2].y, v[3].x, v[3].y);
     } else {
 #pragma unroll
-      for (int c = 0; c < 8; ++c)
-        if (c0 + c < kb) rowp[c] = w[c];
+      for (int q = 0; q < 4; ++q)
+        if (c + q < kb) o[q] = v[q];
     }
     if (!ap) continue;  // the last panel: no trailing matrix
-    store_planes(ap + ((size_t)f * nrow + i) * KW + koff + c0, a_plane, w);
+    store_planes(ap + ((size_t)f * nrow + i) * KW + koff + c, a_plane, v);
     if (i < n) {
 #pragma unroll
-      for (int c = 0; c < 8; ++c) w[c] = cmul_rn(w[c], dinv[c0 + c]);
-      store_planes(bp + ((size_t)f * n + i) * KW + koff + c0, b_plane, w);
+      for (int q = 0; q < 4; ++q) v[q] = cmul_rn(v[q], dinv[c + q]);
+      store_planes(bp + ((size_t)f * n + i) * KW + koff + c, b_plane, v);
     }
   }
 }
