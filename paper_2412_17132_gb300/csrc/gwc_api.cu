@@ -574,10 +574,10 @@ gwc_status enqueue_qp(gwc_ctx* ctx, double* eps_qp, double* dh, int* iters, bool
     LAUNCH(launch_qp_pairs(ctx->d_eps, ctx->d_core_idx, nc, no, ctx->eps_f, ctx->opt.eta, ctx->d_qp, ctx->d_qp_z,
                            ctx->d_qp_active, ctx->d_qp_fac, ctx->d_all_done, ctx->d_active_builds, st));
     TRY(residue_batches(ctx, np, ctx->d_qp_z, ctx->d_qp_rowmap, 1, ctx->d_qp_w, ctx->d_qp_active, st));
-    LAUNCH(launch_qp_assemble_update(ctx->d_eps, ctx->n_states, no, nc, ctx->d_core_idx, ctx->eps_f, ctx->d_xi,
-                                     ctx->d_wxi, ctx->opt.n_im, ctx->d_wim, ctx->d_qp_w, ctx->d_qp_fac, ctx->d_sx,
+    LAUNCH(launch_qp_assemble_update(ctx->d_eps, ctx->n_states, no, nc, ctx->d_core_idx, ctx->d_xi, ctx->d_wxi,
+                                     ctx->opt.n_im, ctx->d_wim, ctx->d_qp_w, ctx->d_qp_fac, ctx->d_sx,
                                      ctx->d_vxc_eff, ctx->opt.qp_tol, ctx->opt.max_qp_iter,
-                                     ctx->opt.qp_mode == GWC_QP_G0W0 ? 1 : 0, ctx->d_qp, ctx->d_all_done, st));
+                                     ctx->opt.qp_mode == GWC_QP_G0W0 ? 1 : 0, ctx->d_qp, ctx->d_all_done, ctx->d_wtmp, st));
     if (poll && (r & 3) == 3) {
       int done = 0;
       CU(cudaMemcpyAsync(&done, ctx->d_all_done, sizeof(int), cudaMemcpyDeviceToHost, st));
@@ -1862,9 +1862,9 @@ gwc_status enqueue_grouped_step(gwc_ctx* const* ctxs, int n, const GroupedPlan& 
   TRY(enqueue_grouped_phase(ctxs, P, P.qp, 1, st, side, ev));
   for (int i = 0; i < n; ++i) {
     gwc_ctx* c = ctxs[i];
-    BCU(launch_qp_assemble_update(c->d_eps, c->n_states, c->n_occ, c->n_core, c->d_core_idx, c->eps_f, c->d_xi, c->d_wxi,
+    BCU(launch_qp_assemble_update(c->d_eps, c->n_states, c->n_occ, c->n_core, c->d_core_idx, c->d_xi, c->d_wxi,
                                   c->opt.n_im, c->d_wim, c->d_qp_w, c->d_qp_fac, c->d_sx, c->d_vxc_eff, c->opt.qp_tol,
-                                  c->opt.max_qp_iter, 0, c->d_qp, c->d_all_done, st));
+                                  c->opt.max_qp_iter, 0, c->d_qp, c->d_all_done, c->d_wtmp, st));
     BCU(launch_qp_finish_hedin(c->d_qp, c->d_eps, c->d_core_idx, c->n_core, c->d_req_eqp, c->d_req_dh, c->d_req_it, st));
   }
   // decoupled Im Sigma on the relative grid and the spectra

@@ -259,11 +259,11 @@ int launch_qp_init(const double* eps, const int* core_idx, int n_core, const int
 int launch_qp_pairs(const double* eps, const int* core_idx, int n_core, int n_occ, double eps_f, double eta,
                     const QpState* st, double* z, int* active, double* fac, int* all_done,
                     unsigned long long* active_count /*+= active pairs, or null*/, cudaStream_t s);
-int launch_qp_assemble_update(const double* eps, int n_states, int n_occ, int n_core, const int* core_idx,
-                              double eps_f, const double* xi, const double* wxi, int n_im, const double* wim,
-                              const double* wpair /*[n_core*n_occ][2]*/, const double* fac, const double* sx,
-                              const double* vxc, double tol, int max_iter, int g0w0, QpState* st, int* all_done,
-                              cudaStream_t s);
+// terms: scratch of n_core * n_states doubles
+int launch_qp_assemble_update(const double* eps, int n_states, int n_occ, int n_core, const int* core_idx, const double* xi,
+                              const double* wxi, int n_im, const double* wim, const double* wpair /*[n_core*n_occ][2]*/,
+                              const double* fac, const double* sx, const double* vxc, double tol, int max_iter, int g0w0,
+                              QpState* st, int* all_done, double* terms, cudaStream_t s);
 // Graphical solutions of the plain G0W0 QP equation on a grid: roots [n_core][max_roots][2] = (w, Z),
 // n_roots [n_core] = number found (may exceed max_roots; only the first max_roots stored).
 int launch_g0w0_scan(const double* omega, int n_w, const double* sigma, const double* eps, const int* core_idx,
