@@ -58,8 +58,8 @@ __global__ void __launch_bounds__(256) ldlt_kernel(S* __restrict__ mats, int n, 
 // The kernel above keeps a matrix on one SM, so a few matrices leave the chip idle (8 of N_aux 1100 in FP64: 279 ms on 8 SMs).
 // Per panel: the diagonal blocks (one CTA per matrix), the rows below (64 per CTA, the factored diagonal read back from the
 // matrix), and the rank-64 update with one 64 x 64 trailing tile per CTA; the arithmetic of every element is the same.
-// Measured in complex FP64: 8 matrices of N_aux 1100, 279 -> 25 ms (update 13.3 ms, of which 12.2 are FP64 multiply-adds at
-// the card's rate; diagonal blocks 6.8 ms, rows 5.1 ms); a batch of 608 matrices of N_aux 200, 18.5 -> 11 ms. FP32 matrices
+// Measured in complex FP64: 8 matrices of N_aux 1100, 279 -> 24 ms (update 13.3 ms, of which 12.2 are FP64 multiply-adds at
+// the card's rate; diagonal blocks 5.6 ms, rows 5.1 ms); a batch of 608 matrices of N_aux 200, 18.5 -> 11 ms. FP32 matrices
 // (the FP32 mode) go the same way.
 template <typename S>
 struct DiagOnlySmem {  // the part of PanelSmem the diagonal needs
@@ -80,7 +80,7 @@ struct DiagOnlySmem {  // the part of PanelSmem the diagonal needs
     dinv2 = dinv1 + NB;
   }
 };
-constexpr int kRowThreads = 64, kDiagThreads = 64;
+constexpr int kRowThreads = 64, kDiagThreads = 128;
 
 template <typename S>
 __global__ void __launch_bounds__(kDiagThreads) ldlt_split_diag_kernel(S* __restrict__ mats, int n, long long ldm, long long stride, int k0,
@@ -286,9 +286,9 @@ __global__ void __launch_bounds__(256) ldlt_solve_kernel(const S* __restrict__ m
 //   solve   the owner of panel k takes its 64 x 64 diagonal block, a warp per right-hand side and two rows per lane (one
 //           exchange per row, no barrier), and puts u into the shared memory of all C CTAs;
 //   update  every CTA subtracts W[rows][panel] u from the rows it owns, W read once through L1.
-// Measured: 8 complex FP32 matrices of N_aux 2450, r = 12, 9.65 -> 0.84 ms; 64 of 1100, r = 6, 2.43 -> 0.29 ms; 8 complex
-// FP64 ones of 1100, 45 -> 2.3 ms. The chain of the n/64 panels bounds it (about 20 us each: 64 exchanges and the cluster
-// barrier). Beyond kFewRhs right-hand sides (the W table, CD-WAC) the kernel above fills the chip.
+// Measured: 8 complex FP32 matrices of N_aux 2450, r = 12, 9.65 -> 0.78 ms; 64 of 1100, r = 6, 2.43 -> 0.29 ms; 8 complex
+// FP64 ones of 1100, 45 -> 2.3 ms. The chain of the n/64 panels bounds it (about 20 us each: 64 exchanges, the cluster
+// barrier and the rows' loads). Beyond kFewRhs right-hand sides (the W table, CD-WAC) the kernel above fills the chip.
 constexpr int kFewRhs = 32;
 constexpr int kFewSmem = 200 * 1024;
 constexpr int FQ = 4;  // right-hand sides per thread of the update
@@ -429,11 +429,16 @@ __global__ void __launch_bounds__(256) ldlt_solve_few_kernel(const S* __restrict
         S a[FQ];
 #pragma unroll
         for (int j = 0; j < FQ; ++j) a[j] = ar[j];
-#pragma unroll 1
-        for (int l0 = 0; l0 < SB; l0 += 4 * PER) {
-          float4 x[4];
+        // the row's next 64 bytes are on their way while the current ones are used
+        constexpr int ST4 = 4 * PER;
+        float4 x[4], y[4];
 #pragma unroll
-          for (int c = 0; c < 4; ++c) x[c] = __ldg(reinterpret_cast<const float4*>(wrow + l0 + c * PER));
+        for (int c = 0; c < 4; ++c) x[c] = __ldg(reinterpret_cast<const float4*>(wrow + c * PER));
+#pragma unroll 1
+        for (int l0 = 0; l0 < SB; l0 += ST4) {
+          const int ln = l0 + ST4 < SB ? l0 + ST4 : l0;
+#pragma unroll
+          for (int c = 0; c < 4; ++c) y[c] = __ldg(reinterpret_cast<const float4*>(wrow + ln + c * PER));
 #pragma unroll
           for (int c = 0; c < 4; ++c) {
             const S* xs = reinterpret_cast<const S*>(&x[c]);
@@ -444,6 +449,8 @@ __global__ void __launch_bounds__(256) ldlt_solve_few_kernel(const S* __restrict
               for (int j = 0; j < FQ; ++j) a[j] = sfnms(xs[e], ul[j], a[j]);
             }
           }
+#pragma unroll
+          for (int c = 0; c < 4; ++c) x[c] = y[c];
         }
 #pragma unroll
         for (int j = 0; j < FQ; ++j) ar[j] = a[j];

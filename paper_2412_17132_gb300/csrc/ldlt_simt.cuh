@@ -276,6 +276,15 @@ __device__ void factor_diag_warp(S (*lkk)[NB + 1], S* dinv, int kb, int& sing) {
 __device__ __forceinline__ double bcast(double v, int l) { return __shfl_sync(0xffffffffu, v, l); }
 __device__ __forceinline__ double2 bcast(double2 v, int l) { return make_double2(bcast(v.x, l), bcast(v.y, l)); }
 
+// 1 / d by a warp that holds the same d in every lane: of the complex reciprocal each half of the warp divides one part (an
+// FP64 division is some twenty dependent instructions)
+__device__ __forceinline__ double sinv_halves(double d) { return sinv(d); }
+__device__ __forceinline__ double2 sinv_halves(double2 d) {
+  const bool h = (threadIdx.x & 16) != 0;
+  const double den = d.x * d.x + d.y * d.y, q = (h ? -d.y : d.x) / den, o = __shfl_xor_sync(0xffffffffu, q, 16);
+  return h ? make_double2(o, q) : make_double2(q, o);
+}
+
 // Columns j .. j + 7 of the block in factor_diag_regs: v[c] = column j + c of the lane's row, CNT columns still in work.
 template <typename S, int CNT>
 __device__ __forceinline__ void factor_diag_cols(S (&v)[NB], S (*lkk)[NB + 1], S* dinv, int j0, int kb, int& sing) {
@@ -285,7 +294,7 @@ __device__ __forceinline__ void factor_diag_cols(S (&v)[NB], S (*lkk)[NB + 1], S
     S d = bcast(v[0], j);
     const bool zero = sabs2(d) < 1e-60;
     if (zero) d = sfrom<S>(1.0, 0.0);
-    const S inv = sinv(d), w = v[0], lij = smul(w, inv);
+    const S inv = sinv_halves(d), w = v[0], lij = smul(w, inv);
     if (i > j) {
       lkk[j][i] = w;  // (above the diagonal: scratch for the row operations of this step)
       lkk[i][j] = lij;
@@ -301,7 +310,7 @@ __device__ __forceinline__ void factor_diag_cols(S (&v)[NB], S (*lkk)[NB + 1], S
 }
 
 // The same factorisation with lane i's row in registers, for FP64: the version above reads and writes every element through
-// shared memory, one after the other (a batch of 608 FP64 matrices, two blocks each: 0.98 ms, in registers 0.58 ms).
+// shared memory, one after the other (a batch of 608 FP64 matrices, two blocks each: 0.98 ms, in registers 0.49 ms).
 template <typename S>
 __device__ void factor_diag_regs(S (*lkk)[NB + 1], S* dinv, int kb, int& sing) {
   const int i = threadIdx.x & 31;
@@ -393,15 +402,19 @@ __device__ void factor_panel_diag(S* __restrict__ A, int n, long long ldm, int k
       }
     }
     grp_sync_n<NT>();
-    // Schur complement of block 2
+    // Schur complement of block 2: its lower triangle, packed over the threads (entries above it are zero)
     for (int e = tid; e < NB * NB; e += NT) {
       const int r = e / NB, c = e % NB;
-      S v = szero<S>();
-      if (r < kb2 && c <= r) {
-        v = A[(long long)(c2 + r) * ldm + (c2 + c)];
+      if (c > r || r >= kb2) ps.lkk2[r][c] = szero<S>();
+    }
+    for (int e = tid; e < kb2 * (kb2 + 1) / 2; e += NT) {
+      int r = (int)((sqrtf(8.f * (float)e + 1.f) - 1.f) * 0.5f);
+      while (r * (r + 1) / 2 > e) --r;
+      while ((r + 1) * (r + 2) / 2 <= e) ++r;
+      const int c = e - r * (r + 1) / 2;
+      S v = A[(long long)(c2 + r) * ldm + (c2 + c)];
 #pragma unroll 8
-        for (int j = 0; j < NB; ++j) v = sfnms(ps.w1s[r][j], ps.l1s[c][j], v);
-      }
+      for (int j = 0; j < NB; ++j) v = sfnms(ps.w1s[r][j], ps.l1s[c][j], v);
       ps.lkk2[r][c] = v;
     }
     grp_sync_n<NT>();
