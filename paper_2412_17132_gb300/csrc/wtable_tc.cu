@@ -223,6 +223,7 @@ __global__ void __launch_bounds__(NTHR, 1) wtable_gemm_kernel(const __grid_const
         float* zl = p.z_lo + ((long long)u * p.b_rows + col0) * TB + rrow;
         for (int cc = 0; cc < TNC / 16 && ok; ++cc) {
           float v[16];
+          double w[16];
           tmem_ld16(lb + cc * 16, v);
 #pragma unroll
           for (int j = 0; j < 16; ++j) {
@@ -231,11 +232,22 @@ __global__ void __launch_bounds__(NTHR, 1) wtable_gemm_kernel(const __grid_const
             const float h = tf32_rn(zz);
             zh[(long long)(cc * 16 + j) * TB] = h;
             zl[(long long)(cc * 16 + j) * TB] = tf32_rn(zz - h);
-            double w = (double)y * (double)y * (double)dinv;
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) w += __shfl_xor_sync(0xffffffffu, w, o);
-            if (lane == 0) red[q * TNC + cc * 16 + j] = w;
+            w[j] = (double)y * (double)y * (double)dinv;
           }
+          // Sums over the warp's rows: half the columns stay with each lane of an exchange, one FP64 addition per element. (A
+          // butterfly per column made five, and at 2 FP64 operations per cycle and SM they bounded the DIAG launches: 33
+          // nodes of N_aux 1190, r = 2040, all GEMMs 2.95 -> 2.15 ms.)
+#pragma unroll
+          for (int o = 16; o > 1; o >>= 1) {
+            const bool up = lane & o;
+#pragma unroll
+            for (int j = 0; j < o / 2; ++j) {
+              const double keep = up ? w[j + o / 2] : w[j], give = up ? w[j] : w[j + o / 2];
+              w[j] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+            }
+          }
+          w[0] += __shfl_xor_sync(0xffffffffu, w[0], 1);
+          if (!(lane & 1)) red[q * TNC + cc * 16 + (lane >> 1)] = w[0];
         }
         // the four epilogue warps meet whatever their wait gave (no warp may skip the barrier)
         asm volatile("bar.sync 1, 128;" ::: "memory");
