@@ -461,8 +461,7 @@ gwc_status enqueue_wim_tail(gwc_ctx* ctx, int k0, int nb, cudaStream_t st) {
     const size_t ebytes = mat_elem_bytes(rk);
     for (int u0 = 0; u0 < nb; u0 += ctx->wim_group) {
       const int ng = std::min(ctx->wim_group, nb - u0);
-      // every node takes the same rows of o_core; one launch for the group (33 nodes of 340 states,
-      // N_aux 1190: 33 launches 0.49 ms, one 0.39 ms)
+      // every node takes the same rows of o_core: one launch for the group converts each row once
       LAUNCH(launch_rhs_gather(rk, ctx->d_o_core, ctx->n_aux, nullptr, 0, ng, r, ctx->n_aux, ctx->d_rhs_im, ctx->ldm,
                                (long long)plane * ctx->ldm, ctx->d_bnorm, st));
       cudaEvent_t evs = ev_begin(ctx, st);

@@ -1,6 +1,8 @@
 // Small element-wise kernels of the self-energy path: transition energies, the
 // frequency factor table D_ia(z), precision copies of O_ov, right-hand-side gathers,
 // the exchange self-energy and output conversion.
+#include <algorithm>
+
 #include "gwc_internal.h"
 
 namespace gwc {
@@ -52,18 +54,21 @@ __global__ void split_o_kernel(const double* __restrict__ o, int n_aux, int n_ov
   f32[t] = (float)v;
 }
 
+// A CTA converts one row for the `share` matrices from blockIdx.y * share on (share > 1: they all take the same row).
 template <typename S>
 __global__ void rhs_gather_kernel(const double* __restrict__ src, long long src_row_stride, const int* __restrict__ row_of,
-                                  int row_f, int r, int n_aux, S* __restrict__ dst, long long ldr, long long rhs_stride,
-                                  double* __restrict__ bnorm2) {
-  int f = blockIdx.y, q = blockIdx.x;
+                                  int row_f, int F, int share, int r, int n_aux, S* __restrict__ dst, long long ldr,
+                                  long long rhs_stride, double* __restrict__ bnorm2) {
+  const int f = blockIdx.y * share, f1 = min(F, f + share), q = blockIdx.x;
   long long row = row_of ? row_of[f * r + q] : (long long)f * row_f + q;
   const double* s = src + (size_t)row * src_row_stride;
   S* d = dst + f * rhs_stride + q * ldr;
   double acc = 0.0;
   for (int p = threadIdx.x; p < n_aux; p += blockDim.x) {
     double v = s[p];
-    d[p] = sfrom<S>(v, 0.0);
+    const S e = sfrom<S>(v, 0.0);
+    S* o = d + p;
+    for (int u = f; u < f1; ++u, o += rhs_stride) *o = e;
     acc += v * v;
   }
   __shared__ double red[32];
@@ -73,7 +78,7 @@ __global__ void rhs_gather_kernel(const double* __restrict__ src, long long src_
   if (threadIdx.x == 0) {
     double t = 0.0;
     for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += red[w];
-    bnorm2[f * r + q] = t;
+    for (int u = f; u < f1; ++u) bnorm2[u * r + q] = t;
   }
 }
 
@@ -178,19 +183,22 @@ int launch_split_o(const double* o_ov, int n_aux, int n_ov, int n_aux_pad, int n
 
 int launch_rhs_gather(MatKind kind, const double* src, long long src_row_stride, const int* row_of, int row_f, int F, int r,
                       int n_aux, void* dst, long long ldr, long long rhs_stride, double* bnorm2, cudaStream_t s) {
-  dim3 g(r, F);
+  // The same rows for every matrix: a CTA writes several copies of what it read (the conversions and the FP64 sum bound a
+  // CTA per copy: 33 nodes of 340 states with 6 cores, N_aux 1190, 394 -> 68 us), as long as some 16 CTAs per SM remain.
+  const int share = (!row_of && row_f == 0) ? std::max(1, (int)std::min<long long>(F, (long long)F * r / (16 * 152))) : 1;
+  dim3 g(r, (F + share - 1) / share);
   switch (kind) {
     case MatKind::RealF32:
-      rhs_gather_kernel<float><<<g, 128, 0, s>>>(src, src_row_stride, row_of, row_f, r, n_aux, (float*)dst, ldr, rhs_stride, bnorm2);
+      rhs_gather_kernel<float><<<g, 128, 0, s>>>(src, src_row_stride, row_of, row_f, F, share, r, n_aux, (float*)dst, ldr, rhs_stride, bnorm2);
       break;
     case MatKind::CplxF32:
-      rhs_gather_kernel<float2><<<g, 128, 0, s>>>(src, src_row_stride, row_of, row_f, r, n_aux, (float2*)dst, ldr, rhs_stride, bnorm2);
+      rhs_gather_kernel<float2><<<g, 128, 0, s>>>(src, src_row_stride, row_of, row_f, F, share, r, n_aux, (float2*)dst, ldr, rhs_stride, bnorm2);
       break;
     case MatKind::RealF64:
-      rhs_gather_kernel<double><<<g, 128, 0, s>>>(src, src_row_stride, row_of, row_f, r, n_aux, (double*)dst, ldr, rhs_stride, bnorm2);
+      rhs_gather_kernel<double><<<g, 128, 0, s>>>(src, src_row_stride, row_of, row_f, F, share, r, n_aux, (double*)dst, ldr, rhs_stride, bnorm2);
       break;
     case MatKind::CplxF64:
-      rhs_gather_kernel<double2><<<g, 128, 0, s>>>(src, src_row_stride, row_of, row_f, r, n_aux, (double2*)dst, ldr, rhs_stride, bnorm2);
+      rhs_gather_kernel<double2><<<g, 128, 0, s>>>(src, src_row_stride, row_of, row_f, F, share, r, n_aux, (double2*)dst, ldr, rhs_stride, bnorm2);
       break;
   }
   return cudaPeekAtLastError() == cudaSuccess ? 1 : -1;
