@@ -276,19 +276,21 @@ __global__ void __launch_bounds__(NTHR, 1) wtable_gemm_kernel(const __grid_const
   }
 }
 
-// W planes: hi / lo TF32 of the strictly lower part of each factored matrix (rows and columns >= n zero).
+// W planes: hi / lo TF32 of the strictly lower part of each factored matrix (rows and columns >= n zero). A CTA per row
+// and node: these conversions move bytes only, and a 64-bit division per element bounded them
+// (33 nodes of N_aux 1190: this 181 -> 101 us, all wt_split_c 367 -> 175 us, widen 129 -> 90 us).
 __global__ void wt_split_w_kernel(const float* __restrict__ mats, long long ldm, long long m_node, int es, int n, int n_pad,
-                                  float* __restrict__ w_hi, float* __restrict__ w_lo, int ng) {
-  const long long per = (long long)n_pad * n_pad;
-  for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < per * ng; e += (long long)gridDim.x * blockDim.x) {
-    const int u = (int)(e / per);
-    const long long f = e - (long long)u * per;
-    const int row = (int)(f / n_pad), col = (int)(f - (long long)row * n_pad);
-    float v = 0.0f;
-    if (row < n && col < row) v = mats[(long long)u * m_node + ((long long)row * ldm + col) * es];
+                                  float* __restrict__ w_hi, float* __restrict__ w_lo) {
+  const int row = blockIdx.x, u = blockIdx.y;
+  const float* m = mats + (long long)u * m_node + (long long)row * ldm * es;
+  const long long o = ((long long)u * n_pad + row) * n_pad;
+  const int end = row < n ? row : 0;  // columns that hold W
+#pragma unroll 4
+  for (int col = threadIdx.x; col < n_pad; col += 256) {
+    const float v = col < end ? m[(long long)col * es] : 0.0f;
     const float h = tf32_rn(v);
-    w_hi[e] = h;
-    w_lo[e] = tf32_rn(v - h);
+    w_hi[o + col] = h;
+    w_lo[o + col] = tf32_rn(v - h);
   }
 }
 
@@ -347,19 +349,26 @@ __global__ void __launch_bounds__(TB) wt_linv_kernel(const float* __restrict__ m
   linv_rows<32>(v, lsm, 96, hi, lo);
 }
 
-// c planes of block i: hi / lo TF32 of the right-hand sides' rows k0 .. k0 + 127 (zero beyond n and r).
+// c planes of block i: hi / lo TF32 of the right-hand sides' rows k0 .. k0 + 127 (zero beyond n and r); a CTA per CC columns
+// of a node.
+constexpr int CC = 8;
 __global__ void wt_split_c_kernel(const float* __restrict__ c, long long ldc, long long c_node, int n, int r, int b_rows,
-                                  int k0, int ng, float* __restrict__ c_hi, float* __restrict__ c_lo) {
-  const long long per = (long long)b_rows * TB;
-  for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < per * ng; e += (long long)gridDim.x * blockDim.x) {
-    const int u = (int)(e / per);
-    const long long f = e - (long long)u * per;
-    const int col = (int)(f / TB), k = (int)(f - (long long)col * TB);
-    float v = 0.0f;
-    if (col < r && k0 + k < n) v = c[(long long)u * c_node + (long long)col * ldc + k0 + k];
-    const float h = tf32_rn(v);
+                                  int k0, float* __restrict__ c_hi, float* __restrict__ c_lo) {
+  const int k = threadIdx.x & (TB - 1), c0 = blockIdx.x * CC + (threadIdx.x >> 7), u = blockIdx.y;
+  const float* src = c + (long long)u * c_node + k0 + k;
+  const long long o = (long long)u * b_rows * TB + k;
+  float v[CC / 2];
+#pragma unroll
+  for (int j = 0; j < CC / 2; ++j) {
+    const int col = c0 + 2 * j;
+    v[j] = col < r && k0 + k < n ? src[(long long)col * ldc] : 0.0f;
+  }
+#pragma unroll
+  for (int j = 0; j < CC / 2; ++j) {
+    const long long e = o + (long long)(c0 + 2 * j) * TB;
+    const float h = tf32_rn(v[j]);
     c_hi[e] = h;
-    c_lo[e] = tf32_rn(v - h);
+    c_lo[e] = tf32_rn(v[j] - h);
   }
 }
 
@@ -373,14 +382,14 @@ __global__ void wt_init_kernel(const double* __restrict__ bnorm, int r, int ng, 
 
 int grid_for(long long n) { return (int)std::min<long long>((n + 255) / 256, 152LL * 16); }
 
-// complex storage (v, 0) of real matrices: dst[u][e] = (src[u][e], 0) for e < per
+// complex storage (v, 0) of real matrices: dst[u][e] = (src[u][e], 0) for e < per, node u = blockIdx.y
 __global__ void widen_kernel(const float* __restrict__ src, long long src_node, float2* __restrict__ dst, long long dst_node,
-                             long long per, int nb) {
-  for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < per * nb; e += (long long)gridDim.x * blockDim.x) {
-    const int u = (int)(e / per);
-    const long long k = e - (long long)u * per;
-    dst[(long long)u * dst_node + k] = make_float2(src[(long long)u * src_node + k], 0.0f);
-  }
+                             long long per) {
+  src += blockIdx.y * src_node;
+  dst += blockIdx.y * dst_node;
+  const long long step = (long long)gridDim.x * blockDim.x;
+#pragma unroll 4
+  for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < per; e += step) dst[e] = make_float2(src[e], 0.0f);
 }
 
 // (P, col, node) view of the right-hand sides [node][col][ldc]: extents n, r, ng; box 128 x 256 x 1, no swizzle
@@ -463,13 +472,12 @@ int launch_wtable_tc(const float* mats, int es, int n, long long ldm, long long 
   p.wait_ns = wait_ns;
 
   wt_init_kernel<<<grid_for((long long)r * ng), 256, 0, s>>>(bnorm, r, ng, table, t_node);
-  wt_split_w_kernel<<<grid_for((long long)n_pad * n_pad * ng), 256, 0, s>>>(mats, ldm, m_node, es, n, n_pad, w_hi, w_lo, ng);
+  wt_split_w_kernel<<<dim3(n_pad, ng), 256, 0, s>>>(mats, ldm, m_node, es, n, n_pad, w_hi, w_lo);
   wt_linv_kernel<<<n_blk * ng, TB, LINV_SMEM, s>>>(mats, ldm, m_node, es, n, n_blk, l_hi, l_lo);
   if (cudaPeekAtLastError() != cudaSuccess) return -1;
   int launches = 3;
   for (int i = 0; i < n_blk; ++i) {
-    wt_split_c_kernel<<<grid_for((long long)r_pad * TB * ng), 256, 0, s>>>(rhs, ldc, c_node, n, r, r_pad, i * TB, ng, c_hi,
-                                                                            c_lo);
+    wt_split_c_kernel<<<dim3(r_pad / CC, ng), 256, 0, s>>>(rhs, ldc, c_node, n, r, r_pad, i * TB, c_hi, c_lo);
     p.mode = 0;
     p.blk = i;
     p.a_hi = l_hi_m;
@@ -499,7 +507,8 @@ int launch_wtable_tc(const float* mats, int es, int n, long long ldm, long long 
 
 int launch_widen_real(const float* src, long long src_node, void* dst, long long dst_node, long long per, int nb,
                       cudaStream_t s) {
-  widen_kernel<<<grid_for(per * nb), 256, 0, s>>>(src, src_node, static_cast<float2*>(dst), dst_node, per, nb);
+  const int x = (int)std::min<long long>((per + 1023) / 1024, (152LL * 16 + nb - 1) / nb);  // four elements a thread, 16 CTAs per SM
+  widen_kernel<<<dim3(std::max(x, 1), nb), 256, 0, s>>>(src, src_node, static_cast<float2*>(dst), dst_node, per);
   return cudaPeekAtLastError() == cudaSuccess ? 1 : -1;
 }
 
