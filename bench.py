@@ -412,7 +412,7 @@ def run_gpu(args):
                 tf32 = peaks.get("bf16_tflops_sustained", peaks.get("bf16_tflops")) * 1.1 / 2.25
                 peak = tf32 / 3.0
                 split = os.environ.get("GWC_FACTOR", "") != "tc"
-                roof = {"kernel": ("ldlt_update_kernel + ldlt_panel_kernel (complex-symmetric LDL^T per 64-column "
+                roof = {"kernel": ("ldlt_update_kernel + ldlt_diag_kernel + ldlt_rows_kernel (complex-symmetric LDL^T per 64-column "
                                    "panel over the batch: tcgen05 3xTF32 updates + SIMT panels)") if split else
                                   ("ldlt_tc_kernel (batched complex-symmetric LDL^T, FP32: tcgen05 3xTF32 trailing "
                                    "updates + SIMT panels)"),

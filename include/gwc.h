@@ -48,7 +48,8 @@ typedef enum {
 
 /* Arithmetic of the polarizability build chi0 and of the dielectric factorisation.
  * All modes keep the self-energy assembly, the QP iteration and the cumulant in FP64.
- *   FP64       : chi0 FP64 (SIMT), factorisation and solves FP64        (plain FP64 path)
+ *   FP64       : chi0 FP64-accurate (exact products of 8-bit digits on the tensor cores; SIMT FP64
+ *                below 64 auxiliary functions), factorisation and solves FP64   (plain FP64 path)
  *   FP32       : chi0 FP32 (SIMT), factorisation and solves FP32
  *   BF16       : chi0 on tcgen05 tensor cores, BF16 operands, FP32 accumulate; factor FP32
  *   BF16X3     : chi0 on tcgen05, split-BF16 operands (hi*hi + hi*lo + lo*hi), FP32
@@ -169,9 +170,9 @@ gwc_status gwc_workspace_bytes(const gwc_system* sys, const gwc_options* opt, in
  * that keep an earlier kernel for A/B comparisons):
  *   - chi0 on CTA pairs (tcgen05 cta_group::2, 256 x 128 tiles) unless gwc_options.chi0_tile = 1;
  *     GWC_CHI0_KERNEL=single sets chi0_tile = 1 (the one-CTA 128 x 128 kernel).
- *   - complex dielectric matrices factored per 64-column panel: one panel launch (one CTA per
- *     matrix) and one batched tcgen05 trailing update over all matrices (3xTF32, FP32-accurate),
- *     panels in pairs with a one-panel lookahead; GWC_FACTOR=tc keeps the one-CTA-per-matrix
+ *   - complex dielectric matrices factored per 64-column panel: the diagonal blocks (one CTA
+ *     per matrix), the rows below (64 per CTA) and one batched tcgen05 trailing update over all
+ *     matrices (3xTF32, FP32-accurate), panels in pairs with a one-panel lookahead; GWC_FACTOR=tc keeps the one-CTA-per-matrix
  *     tensor-core kernel, GWC_FACTOR=simt the FP32 SIMT kernel.
  *   - imaginary-axis W table: real chi0 builds widened into complex storage, the same split
  *     factorisation, and the forward substitution of the 33-node table as tcgen05 3xTF32 GEMMs

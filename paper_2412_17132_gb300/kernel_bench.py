@@ -1,7 +1,7 @@
 """Per-kernel timing of the three dominant kernel groups through the C-ABI, at a chosen width.
 
 The polarizability build (chi0_pair_kernel, or chi0_tc_kernel with GWC_CHI0_KERNEL=single), the
-complex-symmetric factorisation (per 64-column panel: ldlt_panel_kernel, ldlt_planes_kernel and the
+complex-symmetric factorisation (per 64-column panel: ldlt_diag_kernel, ldlt_rows_kernel and the
 batched ldlt_update_kernel; GWC_FACTOR=tc the one-CTA ldlt_tc_kernel) and the W-table forward
 substitution (wtable_gemm_kernel; GWC_WTABLE=simt the SIMT ldlt_solve_kernel) of one context, timed by
 the library's own CUDA events (`profile=True`): `gwc_screen` on `--freqs` complex frequencies
