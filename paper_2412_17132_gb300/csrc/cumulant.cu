@@ -28,7 +28,12 @@ namespace {
 // Its values at the 32 nodes +-s_m cost 2 FMAs per (node, j) (E_j cos and E_j sin of the 16 positive nodes,
 // E_j = c_j e^{-i w_j t_b}), the Chebyshev coefficients a 16 x 16 cosine transform per parity, and every time one
 // 32-term Chebyshev sum: 100 + 48 FMAs per time instead of 6 N_w at N_w = 800, B = 512. FP64 runs at 1/64 of the
-// FP32 rate here, so the FP64 instruction count is what bounds the path. Measured (n_t = 2^16), the whole spectrum with the direct
+// FP32 rate here, so the FP64 instruction count is what bounds the path.
+// The sum over j of c_j comes off at the end, so every time carries an error of a few ulp of sum |c_j|, c_j = q_j beta_j / w_j^2,
+// where the direct sum's c_j (cos w_j t - 1) vanishes with w_j t. A point next to zero (a window's rounding error, 1.1e-16
+// where 0 was meant) would spoil the spectrum: points with |w_j| t_max <= 2^-10 stay out of the blocks and are added time by
+// time as the direct sum adds them, up to MAXN of them, and a core whose other points sum to more than 2^14 (an error above
+// 1e-11) takes the direct sum. Measured (n_t = 2^16), the whole spectrum with the direct
 // sum below and with this: 6.66 and 0.164 ms for one core at 400 points, 26.5 and 0.935 ms for 22 cores; 0.154 and
 // 0.831 ms with the half-length transform.
 constexpr int NP = 32;       // Chebyshev nodes of a block, NH of them positive
@@ -36,24 +41,83 @@ constexpr int NH = NP / 2;
 constexpr int MAXB = 1024;   // times per block, a power of two in NP .. MAXB
 constexpr int MAXG = 4;      // consecutive blocks of one work item
 constexpr int CT = 256;      // threads
+constexpr int MAXN = 8;      // points next to zero of a core on blocks
+constexpr double kNear = 0x1p-10;
+constexpr float kMaxSum = 0x1p14f;
+
+// the bits of |x|, in the order of |x| (integers and FP32 here: at the FP64 rate each comparison of a CTA takes 128 cycles)
+__device__ __forceinline__ long long abs_bits(double x) { return __double_as_longlong(x) & 0x7fffffffffffffffll; }
+// |x| as FP32, rounded down; infinite from 2^128 on and for NaN
+__device__ __forceinline__ float abs_f32(double x) {
+  const int hi = __double2hiint(x) & 0x7fffffff, e = (hi >> 20) - 1023 + 127;
+  return e >= 255 ? __int_as_float(0x7f800000) : e <= 0 ? 0.f : __int_as_float((e << 23) | (hi & 0xfffff) << 3);
+}
+__device__ __forceinline__ bool next_to_zero(double w, long long near_bits) { return abs_bits(w) <= near_bits; }
+
+// (w_j, c_j) of the points next to zero, in the order of the grid
+struct NearPoints {
+  int n;
+  int j[MAXN];
+  double w[MAXN], c[MAXN];
+};
 
 // Times per block for core c's grid: the largest power of two with w_max B dt / 2 <= 8; 0 where not even NP times fit
-// (a grid beyond w_max dt = 1/2, or one that is not finite): that core takes the direct sum. Every thread gets it.
-__device__ int block_times(const double* __restrict__ w, int n_w, int n_t, double dt) {
-  __shared__ double wm[32];
-  double m = 0.0;
-  bool fine = true;
-  for (int j = threadIdx.x; j < n_w; j += blockDim.x) {
-    const double a = fabs(w[j]);
-    fine = fine && a < 1e300;  // false for infinities and NaN
-    m = fmax(m, a);
+// (a grid beyond w_max dt = 1/2, or one that is not finite): that core takes the direct sum. With coef given, 0 also where the
+// points next to zero are too many or the others' coefficients too large (or not finite), and the points next to zero go
+// to `near` (shared memory). CT threads; every one gets the result, the same in every kernel.
+__device__ int block_times(const double* __restrict__ w, const double* __restrict__ coef, int n_w, int n_t, double dt,
+                           NearPoints* near) {
+  __shared__ long long wm[CT / 32];
+  __shared__ float cm[CT / 32];
+  const long long near_bits = abs_bits(kNear / (dt * n_t));
+  if (coef) {
+    if (threadIdx.x == 0) near->n = 0;
+    __syncthreads();
   }
-  if (!fine) m = 1e300;
-  for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
-  if ((threadIdx.x & 31) == 0) wm[threadIdx.x >> 5] = m;
+  long long top = 0;
+  float s = 0.f;
+  for (int j = threadIdx.x; j < n_w; j += CT) {
+    const double a = w[j], c = coef ? coef[j] : 0.0;
+    top = max(top, abs_bits(a));
+    if (abs_bits(c) == 0) continue;
+    if (next_to_zero(a, near_bits)) {
+      const int q = atomicAdd(&near->n, 1);
+      if (q < MAXN) near->j[q] = j;
+    } else {
+      s += abs_f32(c);
+    }
+  }
+  for (int o = 16; o > 0; o >>= 1) {
+    top = max(top, __shfl_xor_sync(0xffffffffu, top, o));
+    s += __shfl_xor_sync(0xffffffffu, s, o);
+  }
+  if ((threadIdx.x & 31) == 0) {
+    wm[threadIdx.x >> 5] = top;
+    cm[threadIdx.x >> 5] = s;
+  }
   __syncthreads();
-  m = 0.0;
-  for (int k = 0; k < (int)(blockDim.x >> 5); ++k) m = fmax(m, wm[k]);
+  s = 0.f;
+  for (int k = 0; k < CT / 32; ++k) {
+    top = max(top, wm[k]);
+    s += cm[k];
+  }
+  const double m = top < abs_bits(1e300) ? __longlong_as_double(top) : 1e300;  // (infinities and NaN lie above)
+  if (coef) {
+    if (near->n > MAXN || !(s <= kMaxSum)) return 0;
+    if (threadIdx.x == 0) {
+      for (int q = 1; q < near->n; ++q)  // the order of the grid, whichever thread came first
+        for (int r = q; r > 0 && near->j[r] < near->j[r - 1]; --r) {
+          const int x = near->j[r];
+          near->j[r] = near->j[r - 1];
+          near->j[r - 1] = x;
+        }
+      for (int q = 0; q < near->n; ++q) {
+        near->w[q] = w[near->j[q]];
+        near->c[q] = coef[near->j[q]];
+      }
+    }
+    __syncthreads();
+  }
   int b = 0;
   for (int t = NP; t <= MAXB && t <= n_t && m * dt * (0.5 * t) <= 8.0; t <<= 1) b = t;
   return b;
@@ -76,7 +140,7 @@ __global__ void __launch_bounds__(CT) cumulant_coef_kernel(const double* __restr
     return;
   }
   const double* w = omega_rel + (size_t)c * n_w;
-  const int b = tab ? block_times(w, n_w, n_t, dt) : 0;
+  const int b = tab ? block_times(w, nullptr, n_w, n_t, dt, nullptr) : 0;
   const int e = blockIdx.x * CT + threadIdx.x, j = e / NH, m = e % NH;
   if (j >= n_w) return;
   const double wj = w[j];
@@ -98,8 +162,9 @@ __global__ void __launch_bounds__(CT) cumulant_coef_kernel(const double* __restr
 // One work item: G consecutive blocks from block b0 of core c (all of its times).
 template <int G>
 __device__ void cumulant_blocks(const double* __restrict__ w, const double* __restrict__ coef, const double* __restrict__ tab,
-                                int n_w, int B, int b0, double dt, double eta, double2 (*es)[CT] /*[MAXG][CT]*/,
-                                double2 (*cf)[NP] /*[MAXG][NP]*/, const double* cosn, double* s0sh, double2* __restrict__ g) {
+                                int n_w, int B, int b0, double dt, long long near_bits, double eta, double2 (*es)[CT] /*[MAXG][CT]*/,
+                                double2 (*cf)[NP] /*[MAXG][NP]*/, const double* cosn, double* s0sh, const NearPoints& near,
+                                double2* __restrict__ g) {
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const double step = B * dt, tc = dt * ((double)b0 * B + 0.5 * (B - 1));  // centre of the first block
   double ar[G], ai[G];
@@ -110,7 +175,7 @@ __device__ void cumulant_blocks(const double* __restrict__ w, const double* __re
     const int j = j0 + tid;
     double2 e = make_double2(0.0, 0.0), r = make_double2(1.0, 0.0);
     if (j < n_w) {
-      const double cj = coef[j];
+      const double cj = next_to_zero(w[j], near_bits) ? 0.0 : coef[j];
       if (cj != 0.0) {
         double sn, cs;
         sincos(w[j] * tc, &sn, &cs);
@@ -204,9 +269,14 @@ __device__ void cumulant_blocks(const double* __restrict__ w, const double* __re
 #pragma unroll
       for (int side = 0; side < 2; ++side) {
         const int k = side ? kc - 1 - q : kc + q;
-        const double re = (side ? er[u] - dr[u] : er[u] + dr[u]) - sum, im = side ? ei[u] - di[u] : ei[u] + di[u];
-        const double mag = exp(re - eta * (dt * k)) * (k == 0 ? 0.5 : 1.0);
+        double re = (side ? er[u] - dr[u] : er[u] + dr[u]) - sum, im = side ? ei[u] - di[u] : ei[u] + di[u];
         double sn, cs;
+        for (int a = 0; a < near.n; ++a) {
+          sincos(near.w[a] * (dt * k), &sn, &cs);
+          re += near.c[a] * (cs - 1.0);
+          im -= near.c[a] * sn;
+        }
+        const double mag = exp(re - eta * (dt * k)) * (k == 0 ? 0.5 : 1.0);
         sincos(im, &sn, &cs);
         g[k] = make_double2(mag * cs, mag * sn);
       }
@@ -224,10 +294,12 @@ __global__ void __launch_bounds__(CT) cumulant_block_kernel(const double* __rest
   __shared__ double2 cf[MAXG][NP];
   __shared__ double cosn[4 * NP];  // cos(pi k / (2 NP))
   __shared__ double s0sh[CT / 32];
+  __shared__ NearPoints near;
   static_assert((CT / 32) * 32 <= CT, "the warps' partial sums fit in es");
   const int c = blockIdx.y;
   const double* w = omega_rel + (size_t)c * n_w;
-  const int B = block_times(w, n_w, n_t, dt);
+  const long long near_bits = abs_bits(kNear / (dt * n_t));
+  const int B = block_times(w, coef + (size_t)c * n_w, n_w, n_t, dt, &near);
   if (B == 0) return;
   if (threadIdx.x < 4 * NP) cosn[threadIdx.x] = cospi(threadIdx.x * (0.5 / NP));
   __syncthreads();
@@ -238,28 +310,29 @@ __global__ void __launch_bounds__(CT) cumulant_block_kernel(const double* __rest
   const long long all = (long long)nb * gridDim.y, want = 4LL * n_sm;
   if (nb >= 4 && all / 4 >= want) {
     for (int b = 4 * blockIdx.x; b < nb; b += 4 * gridDim.x)
-      cumulant_blocks<4>(w, k, t, n_w, B, b, dt, eta, es, cf, cosn, s0sh, o);
+      cumulant_blocks<4>(w, k, t, n_w, B, b, dt, near_bits, eta, es, cf, cosn, s0sh, near, o);
   } else if (nb >= 2 && all / 2 >= want) {
     for (int b = 2 * blockIdx.x; b < nb; b += 2 * gridDim.x)
-      cumulant_blocks<2>(w, k, t, n_w, B, b, dt, eta, es, cf, cosn, s0sh, o);
+      cumulant_blocks<2>(w, k, t, n_w, B, b, dt, near_bits, eta, es, cf, cosn, s0sh, near, o);
   } else {
     for (int b = blockIdx.x; b < nb; b += gridDim.x)
-      cumulant_blocks<1>(w, k, t, n_w, B, b, dt, eta, es, cf, cosn, s0sh, o);
+      cumulant_blocks<1>(w, k, t, n_w, B, b, dt, near_bits, eta, es, cf, cosn, s0sh, near, o);
   }
 }
 
-// The direct sum over the grid, for the cores whose grid does not fit the blocks (all of them without `blocks`). Each thread
+// The direct sum over the grid, for the cores that do not go by blocks (all of them without `blocks`). Each thread
 // takes KT consecutive times: per grid point one sincos at its first time and one for the step w_j dt, then the phase
 // advances by that rotation (the rotation drifts by ~KT ulp over a block).
 constexpr int KT = 32;
 
-__global__ void cumulant_time_kernel(const double* __restrict__ omega_rel, int n_w, const double* __restrict__ coef,
+__global__ void __launch_bounds__(CT) cumulant_time_kernel(const double* __restrict__ omega_rel, int n_w, const double* __restrict__ coef,
                                      int n_core, int n_t, double dt, double eta, int blocks, double2* __restrict__ g) {
   extern __shared__ double sh[];  // [2][n_w]
   double* sw = sh;
   double* sc = sh + n_w;
   const int c = blockIdx.y;
-  if (blocks && block_times(omega_rel + (size_t)c * n_w, n_w, n_t, dt) > 0) return;
+  __shared__ NearPoints near;
+  if (blocks && block_times(omega_rel + (size_t)c * n_w, coef + (size_t)c * n_w, n_w, n_t, dt, &near) > 0) return;
   for (int j = threadIdx.x; j < n_w; j += blockDim.x) {
     sw[j] = omega_rel[(size_t)c * n_w + j];
     sc[j] = coef[(size_t)c * n_w + j];
@@ -398,8 +471,8 @@ int launch_cumulant_spectrum(const double* omega_rel, int n_w, const double* im_
     if (cudaFuncSetAttribute(cumulant_time_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) != cudaSuccess)
       return -1;
   }
-  dim3 g((n_t + 256 * KT - 1) / (256 * KT), n_core);
-  cumulant_time_kernel<<<g, 256, sm, s>>>(omega_rel, n_w, coef, n_core, n_t, dt, eta, table ? 1 : 0, (double2*)work_a);
+  dim3 g((n_t + CT * KT - 1) / (CT * KT), n_core);
+  cumulant_time_kernel<<<g, CT, sm, s>>>(omega_rel, n_w, coef, n_core, n_t, dt, eta, table ? 1 : 0, (double2*)work_a);
   ++launches;
   double2* src = (double2*)work_a;
   double2* dst = (double2*)work_b;
