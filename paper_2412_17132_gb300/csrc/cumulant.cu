@@ -466,9 +466,11 @@ int launch_cumulant_spectrum(const double* omega_rel, int n_w, const double* im_
     cumulant_block_kernel<<<dim3(per, n_core), CT, 0, s>>>(omega_rel, n_w, coef, table, n_t, dt, eta, n_sm, (double2*)work_a);
     ++launches;
   }
-  size_t sm = sizeof(double) * 2 * (size_t)n_w;
-  if (sm > 48 * 1024) {
-    if (cudaFuncSetAttribute(cumulant_time_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) != cudaSuccess)
+  // beyond 48 KB with the kernel's own shared memory (272 bytes), from 3056 grid points on, a larger limit has to be asked for
+  const size_t sm = sizeof(double) * 2 * (size_t)n_w;
+  if (sm > 47 * 1024) {
+    if (cudaFuncSetAttribute(cumulant_time_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             std::max((int)sm, 16 * 8192)) != cudaSuccess)  // (8192 points: the largest grid of the entry points)
       return -1;
   }
   dim3 g((n_t + CT * KT - 1) / (CT * KT), n_core);
