@@ -48,8 +48,10 @@ typedef enum {
 
 /* Arithmetic of the polarizability build chi0 and of the dielectric factorisation.
  * All modes keep the self-energy assembly, the QP iteration and the cumulant in FP64.
- *   FP64       : chi0 FP64-accurate (exact products of 8-bit digits on the tensor cores; SIMT FP64
- *                below 64 auxiliary functions), factorisation and solves FP64   (plain FP64 path)
+ *   FP64       : chi0 FP64-accurate element by element (exact products of 8-bit digits on the tensor
+ *                cores, elements for which these do not reach that summed in FP64; SIMT FP64 below
+ *                64 auxiliary functions, above 200 000 occupied-virtual pairs and where memory is
+ *                short), factorisation and solves FP64                 (plain FP64 path)
  *   FP32       : chi0 FP32 (SIMT), factorisation and solves FP32
  *   BF16       : chi0 on tcgen05 tensor cores, BF16 operands, FP32 accumulate; factor FP32
  *   BF16X3     : chi0 on tcgen05, split-BF16 operands (hi*hi + hi*lo + lo*hi), FP32

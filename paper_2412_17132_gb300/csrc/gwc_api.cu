@@ -252,8 +252,9 @@ size_t per_matrix_bytes(const gwc_system* s, const Sizes& z) {
   return (size_t)s->n_aux * z.ldm * z.elem_c + (size_t)s->n_core * z.ldm * z.elem_c + 2 * (size_t)z.ld_dtab * 8 + 256;
 }
 
-// Workspace of the FP64 polarizability: the scaled operand's digits of a whole batch, at most 1 GiB, at least one 128-row block.
-// (With 256 MB, launches of 90 tiles left SMs idle: 8 frequencies of N_aux 1100 9.3 ms, with 1 GiB 7.0 ms, with 2 GiB 5.9 ms.)
+// Workspace of the FP64 polarizability: the scaled operand's planes of a whole batch, at most 1 GiB, at least one 128-row block.
+// (With 256 MB, launches of 90 tiles left SMs idle: 8 frequencies of N_aux 1100, with eight digits, 9.3 ms, with 1 GiB 7.0 ms, with
+// 2 GiB 5.9 ms.)
 size_t fixed_work_bytes(const Sizes& z, int batch) {
   const size_t all = chi0_fixed_work_bytes(z.n_ov_pad, 2LL * batch * z.n_aux_pad);
   return std::max(chi0_fixed_work_bytes(z.n_ov_pad, 128), std::min(all, (size_t)1 << 30));
@@ -733,7 +734,7 @@ gwc_status gwc_create(gwc_ctx** out, const gwc_system* s, const gwc_options* o, 
     CTRY(dalloc(ctx, &ctx->d_o_lo, np));
     CTRY(dalloc(ctx, &ctx->d_o_f32, np));
   }
-  // (digits of O: 16 bytes per element; a context that cannot have them keeps the SIMT build)
+  // (digits of O: 22 bytes per element; a context that cannot have them keeps the SIMT build)
   if (o->prec == GWC_PREC_FP64 && chi0_fixed_fits(s->n_aux, (long long)n_ov)) {
     ctx->dig_cap = chi0_fixed_digits_bytes(z.n_aux_pad, z.n_ov_pad);
     char* p = nullptr;
