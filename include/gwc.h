@@ -178,7 +178,10 @@ gwc_status gwc_workspace_bytes(const gwc_system* sys, const gwc_options* opt, in
  *     tensor-core kernel, GWC_FACTOR=simt the FP32 SIMT kernel.
  *   - imaginary-axis W table: real chi0 builds widened into complex storage, the same split
  *     factorisation, and the forward substitution of the 33-node table as tcgen05 3xTF32 GEMMs
- *     (explicit inverse of each 128-row diagonal block); GWC_WTABLE=simt keeps the SIMT solve. */
+ *     (explicit inverse of each 128-row diagonal block); GWC_WTABLE=simt keeps the SIMT solve.
+ * In the FP64 mode the tensor-core chi0 takes 22 bytes per element of O_ov and up to 1 GiB of workspace, where these leave
+ * half of the free device memory; else, and with GWC_CHI0_FP64=simt, the context builds chi0 with the (slower) SIMT kernel, as it
+ * does for a system loaded later whose planes do not fit those of the first. */
 gwc_status gwc_create(gwc_ctx** ctx, const gwc_system* sys, const gwc_options* opt, void* stream);
 
 /* Replaces the system of an existing context (serving slots): no device allocation. The new system

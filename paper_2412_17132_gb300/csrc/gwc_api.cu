@@ -289,6 +289,33 @@ int choose_batch(const gwc_system* s, const gwc_options* o, const Sizes& z, int 
   return (int)f;
 }
 
+// FP64 mode: the planes of O (22 bytes per element) and the workspace of the tensor-core polarizability, taken last and only if
+// they leave half of the device's free memory to others: a context that cannot have them keeps the SIMT build.
+// GWC_CHI0_FP64=simt keeps it in any case (A/B measurements).
+void take_digits(gwc_ctx* ctx, const gwc_system* s, const Sizes& z) {
+  const char* env = std::getenv("GWC_CHI0_FP64");
+  if (ctx->opt.prec != GWC_PREC_FP64 || !chi0_fixed_fits(s->n_aux, (long long)ctx->n_ov) || (env && std::strcmp(env, "simt") == 0))
+    return;
+  const size_t dig = chi0_fixed_digits_bytes(z.n_aux_pad, z.n_ov_pad), fx = fixed_work_bytes(z, ctx->batch);
+  size_t freeb = 0, totalb = 0;
+  if (cudaMemGetInfo(&freeb, &totalb) != cudaSuccess || dig + fx > freeb / 2) return;
+  void *d = nullptr, *e = nullptr, *w = nullptr;
+  if (cudaMalloc(&d, dig) != cudaSuccess || cudaMalloc(&e, sizeof(int) * (size_t)z.n_aux_pad) != cudaSuccess ||
+      cudaMalloc(&w, fx) != cudaSuccess) {
+    cudaFree(d);
+    cudaFree(e);
+    cudaGetLastError();  // the failed allocation is not an error of the context
+    return;
+  }
+  ctx->d_o_dig = d;
+  ctx->d_o_ex = static_cast<int*>(e);
+  ctx->d_fx = w;
+  ctx->dig_cap = dig;
+  ctx->ex_cap = (size_t)z.n_aux_pad;
+  ctx->fx_bytes = fx;
+  ctx->chi0_fixed = true;
+}
+
 gwc_status upload(gwc_ctx* ctx, void* dst, const void* src, size_t bytes, int memory, cudaStream_t st) {
   CU(cudaMemcpyAsync(dst, src, bytes, memory == GWC_MEM_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice, st));
   return GWC_OK;
@@ -734,16 +761,6 @@ gwc_status gwc_create(gwc_ctx** out, const gwc_system* s, const gwc_options* o, 
     CTRY(dalloc(ctx, &ctx->d_o_lo, np));
     CTRY(dalloc(ctx, &ctx->d_o_f32, np));
   }
-  // (digits of O: 22 bytes per element; a context that cannot have them keeps the SIMT build)
-  if (o->prec == GWC_PREC_FP64 && chi0_fixed_fits(s->n_aux, (long long)n_ov)) {
-    ctx->dig_cap = chi0_fixed_digits_bytes(z.n_aux_pad, z.n_ov_pad);
-    char* p = nullptr;
-    CTRY(dalloc(ctx, &p, ctx->dig_cap));
-    ctx->d_o_dig = p;
-    CTRY(dalloc(ctx, &ctx->d_o_ex, round_up(s->n_aux, 128)));
-    ctx->ex_cap = (size_t)z.n_aux_pad;
-    ctx->chi0_fixed = true;
-  }
   // imaginary grid
   {
     std::vector<double> x, w;
@@ -771,12 +788,6 @@ gwc_status gwc_create(gwc_ctx** out, const gwc_system* s, const gwc_options* o, 
   ctx->batch_cap = ctx->batch;
   ctx->border_max = std::min(s->n_core, 64);
   ctx->mats_bytes = (size_t)ctx->batch * (s->n_aux + ctx->border_max) * z.ldm * z.elem_c;
-  if (ctx->chi0_fixed) {
-    ctx->fx_bytes = fixed_work_bytes(z, ctx->batch);
-    char* p = nullptr;
-    CTRY(dalloc(ctx, &p, ctx->fx_bytes));
-    ctx->d_fx = p;
-  }
   {
     char* p = nullptr;
     CTRY(dalloc(ctx, &p, ctx->mats_bytes));
@@ -849,6 +860,7 @@ gwc_status gwc_create(gwc_ctx** out, const gwc_system* s, const gwc_options* o, 
     c.bnorm = std::max(wim_rows, (size_t)ctx->batch * s->n_core);
     c.batch = ctx->batch;
   }
+  take_digits(ctx, s, z);
   if (s->eps) {
     CTRY(load_system(ctx, s, st));
     ctx->loaded = true;
