@@ -226,7 +226,7 @@ __device__ __forceinline__ double warp_sum(const double* __restrict__ op, const 
 }
 
 __global__ void __launch_bounds__(FTHREADS, 1) fixed_gemm_kernel(const __grid_constant__ FixedParams p) {
-  extern __shared__ uint8_t smem_raw[];
+  extern __shared__ __align__(16) uint8_t smem_raw[];
   uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   uint64_t* full = reinterpret_cast<uint64_t*>(base + FST * 2 * FTILE);
   uint64_t* empty = full + FST;

@@ -253,7 +253,7 @@ __device__ __forceinline__ bool decode_item(const Chi0PairGroup* gs, int n_group
 template <bool CPLX, bool GROUPED>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
     chi0_pair_kernel(const __grid_constant__ Chi0PairGroup g_own, PairParams p) {
-  extern __shared__ uint8_t smem_raw[];
+  extern __shared__ __align__(16) uint8_t smem_raw[];
   uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   uint8_t* a_ring = base;                           // NS x [hi | lo], 128 rows
   uint8_t* r_ring = a_ring + NS * 2 * ATILE;        // NS x [k 0..31 | k 32..63] FP32, 64 rows

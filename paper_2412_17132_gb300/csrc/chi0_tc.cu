@@ -166,7 +166,7 @@ __device__ __forceinline__ bool decode_item(const Chi0Group* gs, int n_groups, i
 template <bool CPLX, bool GROUPED>
 __global__ void __launch_bounds__(NTHREADS, 1)
     chi0_tc_kernel(const __grid_constant__ Chi0Group g_own, TcParams p) {
-  extern __shared__ uint8_t smem_raw[];
+  extern __shared__ __align__(16) uint8_t smem_raw[];
   uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   uint8_t* b_ring = base;                            // NB_ST x [hi | lo]
   uint8_t* r_ring = b_ring + NB_ST * 2 * TILE;       // NB_ST x [k 0..31 | k 32..63] FP32, swizzled

@@ -118,11 +118,11 @@ struct DiagSmem {
   static constexpr int ELEMS = XR + PW * LDP;
   uint32_t o;
   __device__ __forceinline__ float2& at(int e) const {
-    extern __shared__ uint8_t smem_raw[];
+    extern __shared__ __align__(16) uint8_t smem_raw[];
     return *reinterpret_cast<float2*>(smem_raw + o + e * 8);
   }
   __device__ __forceinline__ float4 pair(int e) const {  // two neighbours, e even
-    extern __shared__ uint8_t smem_raw[];
+    extern __shared__ __align__(16) uint8_t smem_raw[];
     return *reinterpret_cast<const float4*>(smem_raw + o + e * 8);
   }
   __device__ __forceinline__ float2& dm(int i, int c) const { return at(DM + i * LDP + c); }
@@ -366,7 +366,7 @@ struct PanelInv {
   float2 (*ach)[LDP];  // [CH][65] ... the staged rows below the panel after it (aliases dm and xr)
   static constexpr size_t bytes() { return sizeof(float2) * (PW * PW + DiagSmem::DM + (size_t)CH * LDP); }
   __device__ explicit PanelInv(uint8_t* base) {
-    extern __shared__ uint8_t smem_raw[];
+    extern __shared__ __align__(16) uint8_t smem_raw[];
     float2* p = reinterpret_cast<float2*>(base);
     xg = reinterpret_cast<float2(*)[PW]>(p);
     p += PW * PW;
@@ -799,7 +799,7 @@ __device__ void epilogue_role(const TcSmem& sm, uint32_t tmem_base, float2* __re
 // The factorisation of one matrix A (n columns, nrow rows) by one CTA.
 __device__ __forceinline__ void ldlt_tc_matrix(float2* __restrict__ A, int n, int nrow, long long ldm,
                                                unsigned* __restrict__ status, unsigned long long wait_ns) {
-  extern __shared__ uint8_t smem_raw[];
+  extern __shared__ __align__(16) uint8_t smem_raw[];
   TcSmem sm;
   sm.base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   uint64_t* bars = reinterpret_cast<uint64_t*>(sm.base + OPS_BYTES);
@@ -1013,7 +1013,7 @@ __global__ void __launch_bounds__(ROWS_THREADS)
                      float* __restrict__ bp) {
   const int f = blockIdx.y;
   if (active && !active[f]) return;
-  extern __shared__ uint8_t smem_raw[];
+  extern __shared__ __align__(16) uint8_t smem_raw[];
   float2* xg = reinterpret_cast<float2*>(smem_raw);                        // [64][64], then dinv [64]
   float2(*ach)[LDP] = reinterpret_cast<float2(*)[LDP]>(xg + XD);           // [64][65]
   float2* A = mats + f * stride;
@@ -1095,7 +1095,7 @@ __global__ void __launch_bounds__(ROWS_THREADS)
 }
 
 __global__ void __launch_bounds__(UP_THREADS, 2) ldlt_update_kernel(const __grid_constant__ UpParams p) {
-  extern __shared__ uint8_t smem_raw[];
+  extern __shared__ __align__(16) uint8_t smem_raw[];
   uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   uint64_t* full = reinterpret_cast<uint64_t*>(base + UP_STAGE);
   uint64_t* empty = full + 1;

@@ -100,7 +100,7 @@ __device__ __forceinline__ void tma_store_3d(const CUtensorMap* tm, int x, int y
 __device__ __forceinline__ void tma_store_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
 
 __global__ void __launch_bounds__(NTHR, 1) wtable_gemm_kernel(const __grid_constant__ WtParams p) {
-  extern __shared__ uint8_t smem_raw[];
+  extern __shared__ __align__(16) uint8_t smem_raw[];
   uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   uint64_t* full = reinterpret_cast<uint64_t*>(base + NST * STAGE);
   uint64_t* empty = full + NST;
