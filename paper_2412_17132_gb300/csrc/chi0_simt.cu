@@ -36,7 +36,7 @@ template <typename T, typename S, bool CPLX>
 __global__ void __launch_bounds__(256) chi0_simt_kernel(const T* __restrict__ o, int ldo, int n_aux, int n_ov,
                                                          const T* __restrict__ dtab, int ld_dtab, double alpha,
                                                          double beta, S* __restrict__ out, long long ldm,
-                                                         long long mat_stride, int full, const int* __restrict__ active) {
+                                                         long long mat_stride, const int* __restrict__ active) {
   const int f = blockIdx.y;
   if (active && !active[f]) return;
   int ip, iq;
@@ -107,38 +107,37 @@ __global__ void __launch_bounds__(256) chi0_simt_kernel(const T* __restrict__ o,
     for (int y = 0; y < 4; ++y) {
       int p = p0 + ty + 16 * x, q = q0 + tx + 16 * y;
       if (p >= n_aux || q >= n_aux) continue;
-      if (p < q && !full) continue;
+      if (p < q) continue;
       double re = alpha * (double)acc_re[x][y] + (p == q ? beta : 0.0);
       double im = CPLX ? alpha * (double)acc_im[x][y] : 0.0;
       S v = make_out<S>(re, im);
       m[(long long)p * ldm + q] = v;
-      if (full && ip != iq) m[(long long)q * ldm + p] = v;
     }
 }
 
 }  // namespace
 
 int launch_chi0_simt(MatKind kind, const void* o_ov, int ldo, int n_aux, int n_ov, const void* dtab, int ld_dtab, int F,
-                     double alpha, double beta, void* out, long long ldm, long long mat_stride, int full,
+                     double alpha, double beta, void* out, long long ldm, long long mat_stride,
                      const int* active, cudaStream_t s) {
   int nt = (n_aux + kTile - 1) / kTile;
   dim3 g(nt * (nt + 1) / 2, F);
   switch (kind) {
     case MatKind::RealF64:
       chi0_simt_kernel<double, double, false><<<g, 256, 0, s>>>((const double*)o_ov, ldo, n_aux, n_ov, (const double*)dtab,
-                                                               ld_dtab, alpha, beta, (double*)out, ldm, mat_stride, full, active);
+                                                               ld_dtab, alpha, beta, (double*)out, ldm, mat_stride, active);
       break;
     case MatKind::CplxF64:
       chi0_simt_kernel<double, double2, true><<<g, 256, 0, s>>>((const double*)o_ov, ldo, n_aux, n_ov, (const double*)dtab,
-                                                               ld_dtab, alpha, beta, (double2*)out, ldm, mat_stride, full, active);
+                                                               ld_dtab, alpha, beta, (double2*)out, ldm, mat_stride, active);
       break;
     case MatKind::RealF32:
       chi0_simt_kernel<float, float, false><<<g, 256, 0, s>>>((const float*)o_ov, ldo, n_aux, n_ov, (const float*)dtab,
-                                                             ld_dtab, alpha, beta, (float*)out, ldm, mat_stride, full, active);
+                                                             ld_dtab, alpha, beta, (float*)out, ldm, mat_stride, active);
       break;
     case MatKind::CplxF32:
       chi0_simt_kernel<float, float2, true><<<g, 256, 0, s>>>((const float*)o_ov, ldo, n_aux, n_ov, (const float*)dtab,
-                                                             ld_dtab, alpha, beta, (float2*)out, ldm, mat_stride, full, active);
+                                                             ld_dtab, alpha, beta, (float2*)out, ldm, mat_stride, active);
       break;
   }
   return cudaPeekAtLastError() == cudaSuccess ? 1 : -1;

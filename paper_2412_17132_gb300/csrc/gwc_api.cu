@@ -361,13 +361,13 @@ gwc_status load_system(gwc_ctx* ctx, const gwc_system* s, cudaStream_t st) {
 
 // ---- chi0 dispatch ------------------------------------------------------------------------------
 gwc_status run_chi0_any(gwc_ctx* ctx, bool complex_z, int F, const double* d_z, const int* active, void* out,
-                        double alpha, double beta, int full, long long stride, cudaStream_t st) {
+                        double alpha, double beta, long long stride, cudaStream_t st) {
   const int prec = ctx->opt.prec;
   const bool fp64 = prec == GWC_PREC_FP64;
   LAUNCH(launch_dtable(d_z, F, ctx->d_delta, ctx->n_ov, ctx->ld_dtab, !fp64, ctx->d_dtab, st));
   MatKind kind = complex_z ? cplx_kind(ctx) : real_kind(ctx);
   cudaEvent_t ev = ev_begin(ctx, st);
-  if (prec == GWC_PREC_FP64 && ctx->chi0_fixed && !full) {
+  if (prec == GWC_PREC_FP64 && ctx->chi0_fixed) {
     const int n = launch_chi0_fixed(complex_z, ctx->d_o_ov, ctx->d_o_dig, ctx->d_o_ex, ctx->n_aux, ctx->n_aux_pad, ctx->n_ov,
                                     ctx->n_ov_pad, (const double*)ctx->d_dtab, ctx->ld_dtab, F, alpha, beta, out, ctx->ldm, stride,
                                     active, ctx->d_fx, ctx->fx_bytes, ctx->d_status, ctx->wait_ns, st);
@@ -375,10 +375,10 @@ gwc_status run_chi0_any(gwc_ctx* ctx, bool complex_z, int F, const double* d_z, 
     LAUNCH(n);
   } else if (prec == GWC_PREC_FP64) {
     LAUNCH(launch_chi0_simt(kind, ctx->d_o_ov, ctx->n_ov, ctx->n_aux, ctx->n_ov, ctx->d_dtab, ctx->ld_dtab, F, alpha, beta,
-                            out, ctx->ldm, stride, full, active, st));
+                            out, ctx->ldm, stride, active, st));
   } else if (prec == GWC_PREC_FP32) {
     LAUNCH(launch_chi0_simt(kind, ctx->d_o_f32, ctx->n_ov_pad, ctx->n_aux, ctx->n_ov_pad, ctx->d_dtab, ctx->ld_dtab, F,
-                            alpha, beta, out, ctx->ldm, stride, full, active, st));
+                            alpha, beta, out, ctx->ldm, stride, active, st));
   } else {
     // Launch shape of the pair kernel where the options leave it open: with few 64-wide chunks per tile a persistent launch, which
     // keeps TMEM and the barriers and loads the next tile's first chunks under the last one's epilogue, else a CTA pair per
@@ -391,10 +391,6 @@ gwc_status run_chi0_any(gwc_ctx* ctx, bool complex_z, int F, const double* d_z, 
         ctx->d_status, ctx->wait_ns, factor64(prec), st, ctas);
     if (n == -2) return fail(ctx, GWC_ERR_UNSUPPORTED, "tensor-core chi0 not available for this shape/device");
     LAUNCH(n);
-    if (full) {
-      // the tensor-core kernel writes the lower triangle; mirror for a full matrix
-      return fail(ctx, GWC_ERR_UNSUPPORTED, "full-matrix output not supported by the tensor-core path");
-    }
   }
   ev_end(ctx, kClsChi0, ev, st);
   if (!active) {  // masked launches (QP rounds) are counted on the device: only the builds they do
@@ -425,14 +421,14 @@ double factor_flop(int n, bool cplx, int F) {
 }
 
 gwc_status run_chi0(gwc_ctx* ctx, bool complex_z, int F, const double* d_z, const int* active, void* out, double alpha,
-                    double beta, int full, cudaStream_t st) {
-  return run_chi0_any(ctx, complex_z, F, d_z, active, out, alpha, beta, full, (long long)ctx->n_aux * ctx->ldm, st);
+                    double beta, cudaStream_t st) {
+  return run_chi0_any(ctx, complex_z, F, d_z, active, out, alpha, beta, (long long)ctx->n_aux * ctx->ldm, st);
 }
 
 // eps = 1 - Pi into matrices of `stride` elements (room for appended rows)
 gwc_status run_chi0_stride(gwc_ctx* ctx, bool complex_z, int F, const double* d_z, const int* active, void* out,
                            long long stride, cudaStream_t st) {
-  return run_chi0_any(ctx, complex_z, F, d_z, active, out, -1.0, 1.0, 0, stride, st);
+  return run_chi0_any(ctx, complex_z, F, d_z, active, out, -1.0, 1.0, stride, st);
 }
 
 // ---- imaginary-axis W table --------------------------------------------------------------------
@@ -458,10 +454,10 @@ gwc_status enqueue_wim(gwc_ctx* ctx, cudaStream_t st) {
       // real builds behind the nb complex matrices, widened into them (Im = 0) for the tensor-core LDL^T
       const long long per = (long long)ctx->n_aux * ctx->ldm;
       float* real = reinterpret_cast<float*>(static_cast<char*>(ctx->d_mats) + (size_t)nb * per * 8);
-      TRY(run_chi0(ctx, false, nb, ctx->d_zim + 2 * k0, nullptr, real, -1.0, 1.0, 0, st));
+      TRY(run_chi0(ctx, false, nb, ctx->d_zim + 2 * k0, nullptr, real, -1.0, 1.0, st));
       LAUNCH(launch_widen_real(real, per, ctx->d_mats, per, per, nb, st));
     } else {
-      TRY(run_chi0(ctx, false, nb, ctx->d_zim + 2 * k0, nullptr, ctx->d_mats, -1.0, 1.0, 0, st));
+      TRY(run_chi0(ctx, false, nb, ctx->d_zim + 2 * k0, nullptr, ctx->d_mats, -1.0, 1.0, st));
     }
     TRY(enqueue_wim_tail(ctx, k0, nb, st));
   }
@@ -552,7 +548,7 @@ gwc_status residue_batches_buf(gwc_ctx* ctx, int n_pairs, const double* z_dev, c
       LAUNCH(launch_border_w(ck, ctx->d_mats, ctx->n_aux, ctx->ldm, stride, nb, r, ctx->d_bnorm, wout, (long long)r * 2,
                              act, st));
     } else {
-      TRY(run_chi0(ctx, true, nb, z_dev + 2 * (size_t)p0, act, ctx->d_mats, -1.0, 1.0, 0, st));
+      TRY(run_chi0(ctx, true, nb, z_dev + 2 * (size_t)p0, act, ctx->d_mats, -1.0, 1.0, st));
       cudaEvent_t ev = ev_begin(ctx, st);
       LAUNCH(launch_factor(ctx, ck, ctx->d_mats, ctx->n_aux, ctx->n_aux, stride, nb, act, st));
       ev_end(ctx, kClsFactor, ev, st);
@@ -967,7 +963,7 @@ gwc_status gwc_build_chi0(gwc_ctx* ctx, const double* z, int F, double* chi0, vo
   const long long stride = (long long)ctx->n_aux * ctx->ldm;
   for (int f0 = 0; f0 < F; f0 += ctx->batch) {
     int nb = std::min(ctx->batch, F - f0);
-    TRY(run_chi0(ctx, true, nb, z + 2 * (size_t)f0, nullptr, ctx->d_mats, 1.0, 0.0, 0, st));
+    TRY(run_chi0(ctx, true, nb, z + 2 * (size_t)f0, nullptr, ctx->d_mats, 1.0, 0.0, st));
     LAUNCH(launch_mat_to_c128(ck, ctx->d_mats, ctx->n_aux, ctx->ldm, stride, nb,
                               chi0 + (size_t)f0 * ctx->n_aux * ctx->n_aux * 2, st));
   }
@@ -1004,7 +1000,7 @@ gwc_status gwc_screen(gwc_ctx* ctx, const double* z, int F, const double* rhs, i
   const long long stride = (long long)ctx->n_aux * ctx->ldm;
   for (int f0 = 0; f0 < F && res == GWC_OK; f0 += chunk) {
     int nb = std::min(chunk, F - f0);
-    res = run_chi0(ctx, true, nb, z + 2 * (size_t)f0, nullptr, ctx->d_mats, -1.0, 1.0, 0, st);
+    res = run_chi0(ctx, true, nb, z + 2 * (size_t)f0, nullptr, ctx->d_mats, -1.0, 1.0, st);
     if (res != GWC_OK) break;
     cudaEvent_t evf = ev_begin(ctx, st);
     int n1 = launch_factor(ctx, ck, ctx->d_mats, ctx->n_aux, ctx->n_aux, stride, nb, nullptr, st);

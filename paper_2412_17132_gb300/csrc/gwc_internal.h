@@ -116,11 +116,11 @@ inline size_t mat_elem_bytes(MatKind k) {
 int launch_dtable(const double* z, int F, const double* delta, int n_ov, int ld, bool fp32, void* out,
                   cudaStream_t s);
 
-// SIMT chi0: out[f] (type per kind, leading dim ldm) = alpha*Pi(z_f) + beta*I, lower triangle
-// (and the full square if full != 0). dtab from launch_dtable (same precision as the kernel).
+// SIMT chi0: out[f] (type per kind, leading dim ldm) = alpha*Pi(z_f) + beta*I, lower triangle.
+// dtab from launch_dtable (same precision as the kernel).
 int launch_chi0_simt(MatKind kind, const void* o_ov /*double or float [n_aux][ldo]*/, int ldo, int n_aux, int n_ov,
                      const void* dtab, int ld_dtab, int F, double alpha, double beta, void* out, long long ldm,
-                     long long mat_stride, int full, const int* active, cudaStream_t s);
+                     long long mat_stride, const int* active, cudaStream_t s);
 
 // FP64 chi0 from exact products of 8-bit digits on the tensor cores: same output contract as launch_chi0_simt for the FP64
 // kinds, lower triangle only. The digits of O (chi0_fixed_digits_bytes bytes) and the exponents of its rows ([n_aux_pad] ints)
