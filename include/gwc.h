@@ -115,7 +115,8 @@ typedef struct {
                             kernel's work on that tile or matrix, which drains the copies and
                             MMAs it issued, frees its tensor memory and records
                             GWC_ERR_TIMEOUT (reported by gwc_sync); the results of that call
-                            are undefined, and the context stays usable. 0..60000000          */
+                            are undefined, and the context stays usable. 0..60000000. The FP64 mode
+                            waits one second at least: its results do not depend on this     */
   int chi0_ctas;         /* launch shape of the tensor-core polarizability build: 0 chosen by size,
                             one CTA (or CTA pair) per (tile, frequency group) item or, for
                             N_ov up to 16384 on CTA pairs, one per SM; > 0 at most that many

@@ -23,6 +23,7 @@ thread_local std::string g_create_error;
 
 const double kPi = 3.14159265358979323846;
 const size_t kScreenKeep = (size_t)64 << 20;
+const unsigned long long kDefaultWaitNs = 1000000000ull;
 
 gwc_status fail(gwc_ctx* ctx, gwc_status st, const std::string& msg) {
   if (ctx)
@@ -368,9 +369,11 @@ gwc_status run_chi0_any(gwc_ctx* ctx, bool complex_z, int F, const double* d_z, 
   MatKind kind = complex_z ? cplx_kind(ctx) : real_kind(ctx);
   cudaEvent_t ev = ev_begin(ctx, st);
   if (prec == GWC_PREC_FP64 && ctx->chi0_fixed) {
+    // (FP64 contexts take any wait_us, as with the SIMT build, which has no waits)
+    const unsigned long long wait_ns = std::max(ctx->wait_ns, kDefaultWaitNs);
     const int n = launch_chi0_fixed(complex_z, ctx->d_o_ov, ctx->d_o_dig, ctx->d_o_ex, ctx->n_aux, ctx->n_aux_pad, ctx->n_ov,
                                     ctx->n_ov_pad, (const double*)ctx->d_dtab, ctx->ld_dtab, F, alpha, beta, out, ctx->ldm, stride,
-                                    active, ctx->d_fx, ctx->fx_bytes, ctx->d_status, ctx->wait_ns, st);
+                                    active, ctx->d_fx, ctx->fx_bytes, ctx->d_status, wait_ns, st);
     if (n == -2) return fail(ctx, GWC_ERR_UNSUPPORTED, "FP64 tensor-core chi0 not available for this shape/device");
     LAUNCH(n);
   } else if (prec == GWC_PREC_FP64) {
@@ -713,7 +716,7 @@ gwc_status gwc_create(gwc_ctx** out, const gwc_system* s, const gwc_options* o, 
     if (ck && std::strcmp(ck, "single") == 0) ctx->opt.chi0_tile = 1;
     ctx->chi0_pair = ctx->opt.chi0_tile == 0;
   }
-  ctx->wait_ns = o->wait_us > 0 ? 1000ull * (unsigned long long)o->wait_us : 1000000000ull;
+  ctx->wait_ns = o->wait_us > 0 ? 1000ull * (unsigned long long)o->wait_us : kDefaultWaitNs;
   if (o->group_of_core) ctx->h_group.assign(o->group_of_core, o->group_of_core + s->n_core);
   ctx->opt.group_of_core = nullptr;
   Sizes z = sizes_of(s, o);
