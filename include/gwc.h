@@ -120,8 +120,10 @@ typedef struct {
   int chi0_ctas;         /* launch shape of the tensor-core polarizability build: 0 chosen by size,
                             one CTA (or CTA pair) per (tile, frequency group) item or, for
                             N_ov up to 16384 on CTA pairs, one per SM; > 0 at most that many
-                            CTAs, each looping over the items (persistent). gwc_autotune may
-                            change it */
+                            CTAs, each looping over the items (persistent), so that a number
+                            of at least twice the items gives one CTA (pair) per item.
+                            gwc_autotune may change it; the 0 that it chooses is one CTA (pair)
+                            per item                                                          */
   int chi0_tile;         /* tile shape of the tensor-core polarizability build: 0 256 x 128 tiles
                             on CTA pairs (tcgen05 cta_group::2), 1 128 x 128 tiles on one CTA
                             each (less padding of the triangle at small N_aux, a lower MMA rate

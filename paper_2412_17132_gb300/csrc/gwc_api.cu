@@ -387,7 +387,8 @@ gwc_status run_chi0_any(gwc_ctx* ctx, bool complex_z, int F, const double* d_z, 
     // keeps TMEM and the barriers and loads the next tile's first chunks under the last one's epilogue, else a CTA pair per
     // tile. Measured: N_ov 416 x 608 frequencies 233 -> 175 us, 5859 x 64 2149 -> 2074 us, 6099 x 64 2662 -> 2583 us; 25 779
     // x 8 4896 and 4871 us, 89 571 x 2 12.92 and 12.97 ms.
-    const int ctas = ctx->opt.chi0_ctas > 0 ? ctx->opt.chi0_ctas : ctx->chi0_pair && ctx->n_ov_pad <= 16384 ? ctx->n_sm : 0;
+    const bool by_size = ctx->opt.chi0_ctas == 0 && !ctx->chi0_tuned;
+    const int ctas = by_size && ctx->chi0_pair && ctx->n_ov_pad <= 16384 ? ctx->n_sm : ctx->opt.chi0_ctas;
     int n = (ctx->chi0_pair ? launch_chi0_pair : launch_chi0_tc)(
         prec != GWC_PREC_BF16, ctx->d_o_hi, ctx->d_o_lo, ctx->d_o_f32, ctx->n_ov_pad, ctx->n_aux, ctx->n_aux_pad,
         ctx->n_ov_pad, (const float*)ctx->d_dtab, ctx->ld_dtab, F, complex_z, alpha, beta, out, ctx->ldm, stride, active,
@@ -1546,6 +1547,7 @@ gwc_status gwc_autotune(gwc_ctx* ctx, void* stream, int* chosen) {
       ctx->opt.chi0_ctas = it->second.chi0_ctas;
       ctx->opt.chi0_tile = it->second.chi0_tile;
       ctx->chi0_pair = ctx->opt.chi0_tile == 0;
+      ctx->chi0_tuned = tc;
       if (chosen) *chosen = ctx->batch;
       return GWC_OK;
     }
@@ -1568,6 +1570,8 @@ gwc_status gwc_autotune(gwc_ctx* ctx, void* stream, int* chosen) {
   const int np = ctx->req_n_pairs;
   const int saved_ctas = ctx->opt.chi0_ctas, saved_tile = ctx->opt.chi0_tile;
   int best_ctas = saved_ctas, best_tile = saved_tile;
+  bool tuned = ctx->chi0_tuned;
+  ctx->chi0_tuned = tc;  // (so that shape 0 below is the per-item launch)
   for (int f : cands) {
     if (res != GWC_OK || np <= 0) break;
     const int nb = std::min(f, np);
@@ -1591,6 +1595,7 @@ gwc_status gwc_autotune(gwc_ctx* ctx, void* stream, int* chosen) {
         best = f;
         best_ctas = ctx->opt.chi0_ctas;
         best_tile = ctx->opt.chi0_tile;
+        tuned = tc;
       }
     }
     if (nb < f) break;  // fewer pairs than the candidate: larger batches change nothing
@@ -1602,6 +1607,7 @@ gwc_status gwc_autotune(gwc_ctx* ctx, void* stream, int* chosen) {
   ctx->opt.chi0_ctas = best_ctas;
   ctx->opt.chi0_tile = best_tile;
   ctx->chi0_pair = best_tile == 0;
+  ctx->chi0_tuned = tuned;
   if (res != GWC_OK) return res;
   {
     std::lock_guard<std::mutex> lock(g_tune_mutex);

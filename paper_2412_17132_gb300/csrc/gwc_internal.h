@@ -355,6 +355,7 @@ struct gwc_ctx {
   int wim_group = 1;        // imaginary-axis nodes whose solves share one launch
   bool factor_tc = true;    // complex FP32 factorisations on the tensor cores (mixed-precision modes)
   bool chi0_pair = false;   // tensor-core chi0 on CTA pairs (cta_group::2) instead of one CTA per tile
+  bool chi0_tuned = false;  // opt.chi0_ctas is the autotuner's choice: 0 is one CTA (pair) per item, not a choice by size
   bool wtable_tc = false;   // imaginary-axis W-table solves on the tensor cores (else the SIMT forward substitution)
   bool factor_split = false;  // complex FP32 factorisations as panel launches + batched tensor-core updates
   void* d_lp = nullptr;     // their TF32 planes, lp_bytes bytes
