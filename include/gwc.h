@@ -161,7 +161,8 @@ typedef struct gwc_ctx gwc_ctx;
 gwc_status gwc_default_options(gwc_options* o);
 
 /* Device bytes a context of this shape allocates (resident copies + workspace + the
- * per-grid tables for n_omega real frequencies). Host-only; launches nothing. */
+ * per-grid tables for n_omega real frequencies; in the FP64 mode with the tensor-core chi0's
+ * planes, whether or not the device has the room). Host-only; launches nothing. */
 gwc_status gwc_workspace_bytes(const gwc_system* sys, const gwc_options* opt, int n_omega, size_t* bytes);
 
 /* Creates a context on the current device: validates, allocates, copies the system

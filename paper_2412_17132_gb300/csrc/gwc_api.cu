@@ -269,10 +269,10 @@ size_t resident_bytes(const gwc_system* s, const gwc_options* o, const Sizes& z)
   b += (size_t)s->n_states * s->n_core * s->n_aux * 8;              // o_core
   b += (size_t)(o->n_im + 1) * s->n_states * s->n_core * 8;         // W(i xi) table
   b += (size_t)s->n_states * s->n_core * z.ldm * z.elem_r;          // imaginary-axis RHS
-  b += (size_t)s->n_states * s->n_core * (8 + 16 + 4);              // bnorm, w tmp, rowmap
+  b += (size_t)s->n_states * s->n_core * (8 + 16);                  // bnorm, w tmp
   if (o->prec != GWC_PREC_FP64) b += (size_t)z.n_aux_pad * z.n_ov_pad * (2 + 2 + 4);
-  if (o->prec == GWC_PREC_FP64 && chi0_fixed_fits(s->n_aux, (long long)n_ov))
-    b += chi0_fixed_digits_bytes(z.n_aux_pad, z.n_ov_pad) + fixed_work_bytes(z, o->batch > 0 ? o->batch : 512);
+  if (o->prec == GWC_PREC_FP64 && chi0_fixed_shape(s->n_aux, (long long)n_ov))
+    b += chi0_fixed_digits_bytes(z.n_aux_pad, z.n_ov_pad) + fixed_work_bytes(z, o->batch > 0 ? o->batch : 4 * 152);  // (choose_batch)
   return b;
 }
 

@@ -129,7 +129,8 @@ int launch_chi0_simt(MatKind kind, const void* o_ov /*double or float [n_aux][ld
 constexpr int kFixedMinAux = 64;
 size_t chi0_fixed_digits_bytes(int n_aux_pad, int n_ov_pad);
 size_t chi0_fixed_work_bytes(int n_ov_pad, long long rows);
-bool chi0_fixed_fits(int n_aux, long long n_ov);
+bool chi0_fixed_shape(int n_aux, long long n_ov);  // the sizes it takes
+bool chi0_fixed_fits(int n_aux, long long n_ov);   // and the device can run it
 int launch_chi0_digits(const double* o, int n_aux, int n_ov, int n_aux_pad, int n_ov_pad, void* digits, int* ex, cudaStream_t s);
 int launch_chi0_fixed(bool complex_out, const double* o, const void* digits, const int* ex, int n_aux, int n_aux_pad, int n_ov,
                       int n_ov_pad, const double* dtab, int ld_dtab, int F, double alpha, double beta, void* out, long long ldm,
