@@ -253,10 +253,9 @@ def load_traffic(kernel, workload, units_per_launch):
 
 
 def chi0_kernel_info(n_aux, n_ov):
-    """The tensor-core chi0 kernel the library runs (CTA pairs unless GWC_CHI0_KERNEL=single): its name, its
-    traffic key and the ratio of executed MMA work (whole 128 x 128 tiles of the padded lower triangle, the
-    pair kernel's 256 x 128 tiles) to the algorithmic N_aux (N_aux + 1) N_ov per part. The pair tiles are counted
-    as 256-row blocks from row 0; with an odd number of 128-row blocks the kernel launches fewer."""
+    """The tensor-core chi0 kernel the library runs (CTA pairs unless GWC_CHI0_KERNEL=single): its name and the
+    ratio of the MMA work of a lower triangle covered by 256-row blocks from row 0 (the one-CTA kernel: 128 x 128
+    tiles) to the algorithmic N_aux (N_aux + 1) N_ov per part. The pair kernel's launch is chi0_executed_ratio."""
     n_aux_pad = -(-n_aux // 128) * 128
     n_ov_pad = -(-n_ov // 64) * 64
     nqb = n_aux_pad // 128
@@ -266,6 +265,16 @@ def chi0_kernel_info(n_aux, n_ov):
         npb = -(-n_aux_pad // 256)
         tiles, name = 2 * (npb * (npb - 1) + min(2 * npb, nqb)), "chi0_pair_kernel"
     return name, tiles * 128 * 128 * 2 * n_ov_pad / (n_aux * (n_aux + 1.0) * n_ov)
+
+
+def chi0_executed_ratio(n_aux, n_ov):
+    """Executed MMA work of the chi0 kernel the library runs, over the algorithmic N_aux (N_aux + 1) N_ov per part: the
+    pair kernel's 256 x 128 tiles start at any 128-row block, so the Q block q of n takes (n - q + 1) // 2 of them."""
+    nqb = -(-n_aux // 128)
+    if chi0_kernel_info(n_aux, n_ov)[0] != "chi0_pair_kernel":
+        return chi0_kernel_info(n_aux, n_ov)[1]
+    tiles = 2 * sum((nqb - q + 1) // 2 for q in range(nqb))
+    return tiles * 128 * 128 * 2 * (-(-n_ov // 64) * 64) / (n_aux * (n_aux + 1.0) * n_ov)
 
 
 def job_throughput(local_ms, local_units, pg=None, device=None):
@@ -391,7 +400,7 @@ def run_gpu(args):
         # executed tensor-core work per algorithmic flop: the kernel's whole tiles of the padded lower
         # triangle over the padded contraction (64-wide chunks), times the products per split (3 for bf16x3)
         n_ov = mol.n_occ * mol.n_virt
-        kname, tile_ratio = chi0_kernel_info(mol.n_aux, n_ov)
+        kname, tile_ratio = chi0_kernel_info(mol.n_aux, n_ov)[0], chi0_executed_ratio(mol.n_aux, n_ov)
         mma_mult = {"bf16x3": 3.0, "bf16": 1.0}.get(args.prec, 0.0) * tile_ratio
         if chi0_t >= fac_t and args.prec in ("bf16x3", "bf16"):
             peak = peaks.get("bf16_tflops_sustained", peaks.get("bf16_tflops"))
@@ -733,7 +742,7 @@ def run_pentacene_headline(args):
         chi0_t, fac_t = st["chi0_ms"] * 1e-3, st["factor_ms"] * 1e-3
         chi0_alg = st["chi0_flop"] / chi0_t if chi0_t > 0 else 0.0
         n_ov = mol.n_occ * mol.n_virt
-        kname, tile_ratio = chi0_kernel_info(mol.n_aux, n_ov)
+        kname, tile_ratio = chi0_kernel_info(mol.n_aux, n_ov)[0], chi0_executed_ratio(mol.n_aux, n_ov)
         mma_mult = {"bf16x3": 3.0, "bf16x3f64": 3.0, "bf16": 1.0}.get(args.prec, 0.0) * tile_ratio
         peak = peaks.get("bf16_tflops_sustained", peaks.get("bf16_tflops"))
         per_launch = st["chi0_builds"] / max(1, st["chi0_launches"])
