@@ -218,8 +218,8 @@ int launch_border_rows(MatKind kind, void* mats, int n, long long ldm, long long
 int launch_border_w(MatKind kind, const void* mats, int n, long long ldm, long long stride, int F, int r,
                     const double* bnorm2, double* w, long long w_stride, const int* active, cudaStream_t s);
 
-// Right-hand sides: rhs (S type) [F][r][ldr] overwritten by y = L^{-1} b; then
-// w[f][q] = sum_k y_k^2 / d_k - bnorm2[f][q] (FP64 complex out, interleaved).
+// Right-hand sides rhs (S type) [F][r][ldr], y = L^{-1} b; w[f][q] = sum_k y_k^2 / d_k - bnorm2[f][q] (FP64 complex out,
+// interleaved). rhs is scratch: afterwards it holds D^{-1} y, or the b it came with where r <= 32 takes the cluster form.
 int launch_ldlt_solve_w(MatKind kind, const void* mats, int n, long long ldm, long long mat_stride, void* rhs, int r,
                         long long ldr, long long rhs_stride, const double* bnorm2, int F, double* w,
                         long long w_stride, const int* active, cudaStream_t s);
