@@ -29,13 +29,15 @@ namespace {
 // E_j = c_j e^{-i w_j t_b}), the Chebyshev coefficients a 16 x 16 cosine transform per parity, and every time one
 // 32-term Chebyshev sum: 100 + 48 FMAs per time instead of 6 N_w at N_w = 800, B = 512. FP64 runs at 1/64 of the
 // FP32 rate here, so the FP64 instruction count is what bounds the path.
-// The sum over j of c_j comes off at the end, so every time carries an error of a few ulp of sum |c_j|, c_j = q_j beta_j / w_j^2,
-// where the direct sum's c_j (cos w_j t - 1) vanishes with w_j t. A point next to zero (a window's rounding error, 1.1e-16
-// where 0 was meant) would spoil the spectrum: points with |w_j| t_max <= 2^-10 stay out of the blocks and are added time by
-// time as the direct sum adds them, up to MAXN of them, and a core whose other points sum to more than 2^14 (an error above
-// 1e-11) takes the direct sum. Measured (n_t = 2^16), the whole spectrum with the direct
-// sum below and with this: 6.66 and 0.164 ms for one core at 400 points, 26.5 and 0.935 ms for 22 cores; 0.154 and
-// 0.831 ms with the half-length transform.
+// The coefficients c_j = q_j beta_j / w_j^2 grow without bound towards w = 0 while c_j (e^{-i w_j t} - 1) does not, so nothing may
+// be formed as sum c_j e^{-i w_j t} - sum c_j. With p_j = c_j (e^{-i w_j t_b} - 1) from half angles (-2 c_j sin^2, -2 c_j sin cos),
+//   sum_j c_j (e^{-i w_j t} - 1) = sum_j p_j + sum_j E_j (cos(w_j h s) - 1) - i sum_j E_j sin(w_j h s),  E_j = p_j + c_j,
+// whose terms are all of the size of what they add; the first sum belongs to the block. (Formed with the difference, every time
+// carried a few ulp of sum |c_j|: 1e-11 of the peak at 1.6e4, which a grid point within 3e-4 Ha of zero gives.)
+// Points next to zero (a window's rounding error, 1.1e-16 where 0 was meant), |w_j| t_max <= 2^-10, stay out of the blocks and
+// are added time by time as the direct sum adds them, up to MAXN of them; a core with more, or whose other coefficients sum
+// to more than 2^30, takes the direct sum. Measured (n_t = 2^16), the whole spectrum with the direct
+// sum below and with this: 6.66 and 0.154 ms for one core at 400 points, 26.5 and 0.831 ms for 22 cores.
 constexpr int NP = 32;       // Chebyshev nodes of a block, NH of them positive
 constexpr int NH = NP / 2;
 constexpr int MAXB = 1024;   // times per block, a power of two in NP .. MAXB
@@ -43,7 +45,7 @@ constexpr int MAXG = 4;      // consecutive blocks of one work item
 constexpr int CT = 256;      // threads
 constexpr int MAXN = 8;      // points next to zero of a core on blocks
 constexpr double kNear = 0x1p-10;
-constexpr float kMaxSum = 0x1p14f;
+constexpr float kMaxSum = 0x1p30f;
 
 // the bits of |x|, in the order of |x| (integers and FP32 here: at the FP64 rate each comparison of a CTA takes 128 cycles)
 __device__ __forceinline__ long long abs_bits(double x) { return __double_as_longlong(x) & 0x7fffffffffffffffll; }
@@ -124,7 +126,7 @@ __device__ int block_times(const double* __restrict__ w, const double* __restric
 }
 
 // coef[c][j] = q_j beta_j / w_j^2 with trapezoid weights q_j of the per-core grid, and (tab given, core on blocks)
-// tab[c][j][m] = cos(w_j h s_m), tab[c][j][NH + m] = sin(w_j h s_m), s_m = cos(pi (2 m + 1) / (2 NP)). The last row of the grid
+// tab[c][j][m] = cos(w_j h s_m) - 1, tab[c][j][NH + m] = sin(w_j h s_m), s_m = cos(pi (2 m + 1) / (2 NP)). The last row of the grid
 // writes the transform's factors tw[m] = e^{+2 pi i m / n_t}, m < n_t / 2.
 __global__ void __launch_bounds__(CT) cumulant_coef_kernel(const double* __restrict__ omega_rel, int n_w,
                                                             const double* __restrict__ im_sigma, int n_t, double dt,
@@ -153,45 +155,52 @@ __global__ void __launch_bounds__(CT) cumulant_coef_kernel(const double* __restr
   }
   if (b == 0) return;
   double sn, cs;
-  sincos(wj * ((0.5 * b * dt) * cospi((2 * m + 1) * (0.5 / NP))), &sn, &cs);
+  sincos(0.5 * (wj * ((0.5 * b * dt) * cospi((2 * m + 1) * (0.5 / NP)))), &sn, &cs);
   double* o = tab + ((size_t)c * n_w + j) * NP;
-  o[m] = cs;
-  o[NH + m] = sn;
+  o[m] = -2.0 * sn * sn;
+  o[NH + m] = 2.0 * sn * cs;
 }
 
 // One work item: G consecutive blocks from block b0 of core c (all of its times).
 template <int G>
 __device__ void cumulant_blocks(const double* __restrict__ w, const double* __restrict__ coef, const double* __restrict__ tab,
                                 int n_w, int B, int b0, double dt, long long near_bits, double eta, double2 (*es)[CT] /*[MAXG][CT]*/,
-                                double2 (*cf)[NP] /*[MAXG][NP]*/, const double* cosn, double* s0sh, const NearPoints& near,
+                                double2 (*cf)[NP] /*[MAXG][NP]*/, const double* cosn, double2 (*s0sh)[CT / 32] /*[MAXG][CT / 32]*/, const NearPoints& near,
                                 double2* __restrict__ g) {
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const double step = B * dt, tc = dt * ((double)b0 * B + 0.5 * (B - 1));  // centre of the first block
   double ar[G], ai[G];
+  double2 s0[G];  // sum_j p_j of every block
 #pragma unroll
-  for (int u = 0; u < G; ++u) ar[u] = ai[u] = 0.0;
-  double s0 = 0.0;
+  for (int u = 0; u < G; ++u) {
+    ar[u] = ai[u] = 0.0;
+    s0[u] = make_double2(0.0, 0.0);
+  }
   for (int j0 = 0; j0 < n_w; j0 += CT) {
     const int j = j0 + tid;
-    double2 e = make_double2(0.0, 0.0), r = make_double2(1.0, 0.0);
+    double2 p = make_double2(0.0, 0.0), r = make_double2(0.0, 0.0);  // p_j; e^{-i w_j B dt} - 1
+    double cj = 0.0;
     if (j < n_w) {
-      const double cj = next_to_zero(w[j], near_bits) ? 0.0 : coef[j];
+      cj = next_to_zero(w[j], near_bits) ? 0.0 : coef[j];
       if (cj != 0.0) {
         double sn, cs;
-        sincos(w[j] * tc, &sn, &cs);
-        e = make_double2(cj * cs, -cj * sn);
+        sincos(0.5 * (w[j] * tc), &sn, &cs);
+        const double a = -2.0 * (cj * sn);
+        p = make_double2(a * sn, a * cs);
         if (G > 1) {
-          sincos(w[j] * step, &sn, &cs);
-          r = make_double2(cs, -sn);
+          sincos(0.5 * (w[j] * step), &sn, &cs);
+          r = make_double2(-2.0 * sn * sn, -2.0 * sn * cs);
         }
       }
-      s0 += cj;
     }
     __syncthreads();  // the previous chunk (or item) has been read
 #pragma unroll
     for (int u = 0; u < G; ++u) {
+      const double2 e = make_double2(p.x + cj, p.y);
       es[u][tid] = e;
-      if (u + 1 < G) e = make_double2(e.x * r.x - e.y * r.y, e.x * r.y + e.y * r.x);
+      s0[u].x += p.x;
+      s0[u].y += p.y;
+      if (u + 1 < G) p = make_double2(fma(e.x, r.x, fma(-e.y, r.y, p.x)), fma(e.x, r.y, fma(e.y, r.x, p.y)));
     }
     __syncthreads();
     const int jn = min(CT, n_w - j0);
@@ -207,13 +216,19 @@ __device__ void cumulant_blocks(const double* __restrict__ w, const double* __re
       }
     }
   }
-  // sums over the warps (es holds them), then the node values and sum_j c_j
+  // sums over the warps (es holds them), then the node values and sum_j p_j
   __syncthreads();
   double2* part = &es[0][0];  // [warp][u][node]
 #pragma unroll
   for (int u = 0; u < G; ++u) part[(warp * G + u) * 32 + lane] = make_double2(ar[u], ai[u]);
-  for (int o = 16; o > 0; o >>= 1) s0 += __shfl_down_sync(0xffffffffu, s0, o);
-  if (lane == 0) s0sh[warp] = s0;
+#pragma unroll
+  for (int u = 0; u < G; ++u) {
+    for (int o = 16; o > 0; o >>= 1) {
+      s0[u].x += __shfl_down_sync(0xffffffffu, s0[u].x, o);
+      s0[u].y += __shfl_down_sync(0xffffffffu, s0[u].y, o);
+    }
+    if (lane == 0) s0sh[u][warp] = s0[u];
+  }
   __syncthreads();
   for (int e = tid; e < G * 32; e += CT) {
     double2 a = part[e];
@@ -226,7 +241,7 @@ __device__ void cumulant_blocks(const double* __restrict__ w, const double* __re
     part[e] = a;  // read by this thread alone so far
   }
   __syncthreads();
-  // Chebyshev coefficients: even ones from E cos, odd ones from -i E sin
+  // Chebyshev coefficients: even ones from E (cos - 1), with sum_j p_j on the constant, odd ones from -i E sin
   for (int e = tid; e < G * NP; e += CT) {
     const int u = e / NP, p = e % NP;
     const double2* v = part + u * 32 + (p & 1) * NH;
@@ -238,11 +253,19 @@ __device__ void cumulant_blocks(const double* __restrict__ w, const double* __re
       a.y = fma(v[m].y, k, a.y);
     }
     const double f = p == 0 ? 2.0 / NP : 4.0 / NP;
-    cf[u][p] = (p & 1) ? make_double2(f * a.y, -f * a.x) : make_double2(f * a.x, f * a.y);
-  }
-  double sum = 0.0;
+    a = (p & 1) ? make_double2(f * a.y, -f * a.x) : make_double2(f * a.x, f * a.y);
+    if (p == 0) {
+      double2 s = s0sh[u][0];
 #pragma unroll
-  for (int k = 0; k < CT / 32; ++k) sum += s0sh[k];
+      for (int k = 1; k < CT / 32; ++k) {
+        s.x += s0sh[u][k].x;
+        s.y += s0sh[u][k].y;
+      }
+      a.x += s.x;
+      a.y += s.y;
+    }
+    cf[u][p] = a;
+  }
   __syncthreads();
   for (int q = tid; q < B / 2; q += CT) {  // the times at +-s of every block
     const double s = (2 * q + 1) / (double)B;
@@ -269,7 +292,7 @@ __device__ void cumulant_blocks(const double* __restrict__ w, const double* __re
 #pragma unroll
       for (int side = 0; side < 2; ++side) {
         const int k = side ? kc - 1 - q : kc + q;
-        double re = (side ? er[u] - dr[u] : er[u] + dr[u]) - sum, im = side ? ei[u] - di[u] : ei[u] + di[u];
+        double re = side ? er[u] - dr[u] : er[u] + dr[u], im = side ? ei[u] - di[u] : ei[u] + di[u];
         double sn, cs;
         for (int a = 0; a < near.n; ++a) {
           sincos(near.w[a] * (dt * k), &sn, &cs);
@@ -293,7 +316,7 @@ __global__ void __launch_bounds__(CT) cumulant_block_kernel(const double* __rest
   __shared__ double2 es[MAXG][CT];
   __shared__ double2 cf[MAXG][NP];
   __shared__ double cosn[4 * NP];  // cos(pi k / (2 NP))
-  __shared__ double s0sh[CT / 32];
+  __shared__ double2 s0sh[MAXG][CT / 32];
   __shared__ NearPoints near;
   static_assert((CT / 32) * 32 <= CT, "the warps' partial sums fit in es");
   const int c = blockIdx.y;
