@@ -289,6 +289,7 @@ __global__ void __launch_bounds__(256) ldlt_solve_kernel(const S* __restrict__ m
 // Measured: 8 complex FP32 matrices of N_aux 2450, r = 12, 9.65 -> 0.78 ms; 64 of 1100, r = 6, 2.43 -> 0.29 ms; 8 complex
 // FP64 ones of 1100, 45 -> 2.3 ms. The chain of the n/64 panels bounds it (about 20 us each: 64 exchanges, the cluster
 // barrier and the rows' loads). Beyond kFewRhs right-hand sides (the W table, CD-WAC) the kernel above fills the chip.
+// (Which cluster, and where the kernel above stays: few_ctas.)
 constexpr int kFewRhs = 32;
 constexpr int kFewSmem = 200 * 1024;
 constexpr int FQ = 4;  // right-hand sides per thread of the update
@@ -483,6 +484,46 @@ __global__ void __launch_bounds__(256) ldlt_solve_few_kernel(const S* __restrict
   }
 }
 
+template <typename S>
+size_t few_bytes(int n, int r, int C) {
+  const int np = (n + SB - 1) / SB, rp = (r + FQ - 1) / FQ * FQ;
+  return few_elems((np + C - 1) / C, rp) * sizeof(S) + (size_t)C * r * 16;
+}
+
+int sm_count() {
+  int dev = 0, n = 1;
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 1;
+  return n;
+}
+
+// CTAs per cluster for F matrices, 0 for the one-CTA kernel. Both were measured for real and complex, FP32 and FP64, n 65 .. 1100, r 6
+// .. 32 and 1 to 608 matrices with every cluster size:
+//   the cluster grows until every SM has a CTA; where the arithmetic of a CTA fills an SM (FP64 beyond 8 right-hand sides, complex
+//   FP32 beyond 16), while all of them still run at once (33 complex FP32 matrices of n 416, r = 32: 479 us with 8 CTAs each, 168
+//   with 4, 446 with the kernel above; 64 real FP64 ones of 192, r = 24: 753 us with 4, 401 with 2, 428), and more where
+//   the sums need the room. Up to two panels a second CTA has next to nothing to do.
+//   Beyond 16 right-hand sides a panel's block is work for the one SM that solves it. FP64: one round of such CTAs takes (1.2 +
+//   n / 208) (complex) or (2.45 + n / 300) (real) of what one round of the other kernel takes per panel (1 complex matrix, r = 24: n
+//   65 776 against 616 us, n 192 1320 against 1835, n 416 3340 against 7630). FP32: three rounds of clusters of four and more
+//   lose (152 complex ones of 1100, r = 32: 3270 against 2490 us).
+// At none of the 600 points this is more than 5 % slower than the one-CTA kernel.
+template <typename S>
+int few_ctas(int n, int r, int F) {
+  constexpr bool fp64 = sizeof(typename ST<S>::R) == 8, cplx = ST<S>::kComplex;
+  const int np = (n + SB - 1) / SB, sms = sm_count();
+  const bool full = sizeof(S) >= 8 && r > (fp64 ? 8 : 16);
+  int C = 1;
+  while (C < 8 && C < np - 1 && (full ? 2LL * F * C <= sms : (long long)F * C < sms)) C <<= 1;
+  while (C <= 8 && few_bytes<S>(n, r, C) > (size_t)kFewSmem) C <<= 1;
+  if (C > 8) return 0;
+  if (r > 16) {
+    const double rounds = (double)(((long long)F * C + sms - 1) / sms), other = (double)((F + sms - 1) / sms);
+    if (fp64 && rounds * (cplx ? 1.2 + n / 208.0 : 2.45 + n / 300.0) > other * n / SB) return 0;
+    if (!fp64 && C > 2 && (long long)F * C > 3LL * sms) return 0;
+  }
+  return C;
+}
+
 template <typename S, int QW>
 int run_solve_few(const S* mats, int n, long long ldm, long long stride, const S* rhs, int r, long long ldr,
                   long long rhs_stride, const double* bnorm2, int F, double* w, long long w_stride, const int* active, int C,
@@ -534,15 +575,11 @@ template <typename S>
 int run_solve(const S* mats, int n, long long ldm, long long stride, S* rhs, int r, long long ldr, long long rhs_stride,
               const double* bnorm2, int F, double* w, long long w_stride, const int* active, cudaStream_t s) {
   if (r <= kFewRhs && ldm % 4 == 0 && stride % 4 == 0 && (reinterpret_cast<uintptr_t>(mats) & 15) == 0) {  // 16-byte loads
-    // the smallest cluster that gives every SM a CTA (F C >= 148 .. 160 on these parts), more where the sums need the room
-    const int np = (n + SB - 1) / SB, rp = (r + FQ - 1) / FQ * FQ;
-    for (int C = 1; C <= 8; C <<= 1) {
-      const size_t few = few_elems((np + C - 1) / C, rp) * sizeof(S) + (size_t)C * r * 16;
-      if (few > (size_t)kFewSmem || (C < 8 && C < np && F * C < 152)) continue;
-      if (r <= 8) return run_solve_few<S, 1>(mats, n, ldm, stride, rhs, r, ldr, rhs_stride, bnorm2, F, w, w_stride, active, C, few, s);
-      if (r <= 16) return run_solve_few<S, 2>(mats, n, ldm, stride, rhs, r, ldr, rhs_stride, bnorm2, F, w, w_stride, active, C, few, s);
-      return run_solve_few<S, 4>(mats, n, ldm, stride, rhs, r, ldr, rhs_stride, bnorm2, F, w, w_stride, active, C, few, s);
-    }
+    const int C = few_ctas<S>(n, r, F);
+    const size_t few = C ? few_bytes<S>(n, r, C) : 0;
+    if (C && r <= 8) return run_solve_few<S, 1>(mats, n, ldm, stride, rhs, r, ldr, rhs_stride, bnorm2, F, w, w_stride, active, C, few, s);
+    if (C && r <= 16) return run_solve_few<S, 2>(mats, n, ldm, stride, rhs, r, ldr, rhs_stride, bnorm2, F, w, w_stride, active, C, few, s);
+    if (C) return run_solve_few<S, 4>(mats, n, ldm, stride, rhs, r, ldr, rhs_stride, bnorm2, F, w, w_stride, active, C, few, s);
   }
   static bool attr = false;
   const size_t sm = solve_smem<S>();
