@@ -12,7 +12,7 @@
 //   diagonal             d
 //   strictly upper part  L^T       (A[j][i] = L_ij; scratch used by the trailing updates)
 //
-// Right-looking and blocked, by one CTA per matrix (a single panel) or as launches over all matrices (below):
+// Right-looking and blocked, by one CTA per matrix or as launches over all matrices (below):
 //   * 64-wide panels, each factored as two 32-wide halves: the two 32 x 32 diagonal blocks in
 //     shared memory, then every row below in one pass by one thread (solve against block 1,
 //     apply block 1 to its block-2 columns, solve against block 2), storing W (lower) and L
@@ -55,12 +55,12 @@ __global__ void __launch_bounds__(256) ldlt_kernel(S* __restrict__ mats, int n, 
 }
 
 // ---- the same factorisation over all SMs ------------------------------------------------------------
-// The kernel above keeps a matrix on one SM, so a few matrices leave the chip idle (8 of N_aux 1100 in FP64: 279 ms on 8 SMs).
+// The kernel above keeps a matrix on one SM, so a few large matrices leave the chip idle (8 of N_aux 1100 in FP64: 279 ms on 8 SMs).
 // Per panel: the diagonal blocks (one CTA per matrix), the rows below (64 per CTA, the factored diagonal read back from the
 // matrix), and the rank-64 update with one 64 x 64 trailing tile per CTA; the arithmetic of every element is the same.
 // Measured in complex FP64: 8 matrices of N_aux 1100, 279 -> 24 ms (update 13.3 ms, of which 12.2 are FP64 multiply-adds at
-// the card's rate; diagonal blocks 5.6 ms, rows 5.1 ms); a batch of 608 matrices of N_aux 200, 18.5 -> 11 ms. FP32 matrices
-// (the FP32 mode) go the same way.
+// the card's rate; diagonal blocks 5.6 ms, rows 5.1 ms); a batch of 608 matrices of N_aux 200, 18.5 -> 11 ms. Which
+// of the two: one_cta_factor.
 template <typename S>
 struct DiagOnlySmem {  // the part of PanelSmem the diagonal needs
   S (*lkk1)[NB + 1];
@@ -556,11 +556,27 @@ size_t solve_smem() {
   return SolveSmem<S>::bytes();
 }
 
+// Whether F matrices go by one CTA each. They do with a single panel, which has no update, and where they all run at once (two per
+// SM, one in complex FP64) and either the chain of a small matrix's panels is shorter inside one CTA than as launches, up to n0, or
+// there are so many that they fill the chip: the launches' time grows with F n^3, the other does not grow. The line is F =
+// slots (1 - (n0 / n)^2). Measured (real and complex, FP32 and FP64, n 65 .. 1100, 1 to 608 matrices; launches against one CTA, us):
+// complex FP32 n 96 F 64 146 and 125, n 320 F 152 691 and 651, F 33 558 and 612; real FP64 n 128 F 64 400 and 348, n 256 F 152
+// 1447 and 1261, F 33 1053 and 1253; real FP32 n 200 F 152 316 and 247. Nowhere more than 4 % slower
+// than one CTA per matrix, 12 % than the launches.
+template <typename S>
+bool one_cta_factor(int n, int F) {
+  if (n <= PW) return true;
+  constexpr bool fp64 = sizeof(typename ST<S>::R) == 8, cplx = ST<S>::kComplex;
+  const int n0 = fp64 ? (cplx ? 128 : 160) : (cplx ? 192 : 256), sms = sm_count();
+  const int slots = F <= sms || (fp64 && cplx) ? sms : 2 * sms;
+  return F <= slots && (n <= n0 || (double)F * n * n >= (double)slots * ((double)n * n - (double)n0 * n0));
+}
+
 template <typename S>
 int run_ldlt(S* mats, int n, int nrow, long long ldm, long long stride, int F, const int* active, unsigned* status,
              cudaStream_t s) {
-  // one panel has no update, and a batch beyond the grid's y extent stays with the kernel above
-  if (n > PW && F <= 65535) return run_ldlt_split(mats, n, nrow, ldm, stride, F, active, status, s);
+  // a batch beyond the grid's y extent stays with the kernel above
+  if (!one_cta_factor<S>(n, F) && F <= 65535) return run_ldlt_split(mats, n, nrow, ldm, stride, F, active, status, s);
   static bool attr = false;
   const size_t sm = std::max(FactorSmem<S>::bytes(), PanelSmem<S, kSimtThreads>::bytes());
   if (!attr) {
