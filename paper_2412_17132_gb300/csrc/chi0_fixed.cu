@@ -438,7 +438,7 @@ size_t chi0_fixed_work_bytes(int n_ov_pad, long long rows) {
   return (size_t)rows * ((size_t)n_ov_pad * 2 * NPL + sizeof(int)) + 1024;
 }
 
-bool chi0_fixed_shape(int n_aux, long long n_ov) { return n_aux >= kFixedMinAux && n_ov <= kMaxOv; }
+bool chi0_fixed_shape(int n_aux, long long n_ov) { return n_aux >= kFixedMinAux && n_ov >= kFixedMinOv && n_ov <= kMaxOv; }
 bool chi0_fixed_fits(int n_aux, long long n_ov) { return chi0_fixed_shape(n_aux, n_ov) && tc_supported(); }
 
 int launch_chi0_digits(const double* o, int n_aux, int n_ov, int n_aux_pad, int n_ov_pad, void* digits, int* ex,

@@ -1,5 +1,5 @@
 // SIMT polarizability build: the FP32 mode, and in the FP64 mode what the exact digit products of chi0_fixed.cu do not
-// take (few auxiliary functions, very long contractions, no room for the digits).
+// take (few auxiliary functions, very short or very long contractions, no room for the digits).
 //
 //   Pi_PQ(z_f) = sum_k O_Pk D_f(k) O_Qk,   k = (i, a) occupied-virtual pair
 //

@@ -126,7 +126,10 @@ int launch_chi0_simt(MatKind kind, const void* o_ov /*double or float [n_aux][ld
 // kinds, lower triangle only. The digits of O (chi0_fixed_digits_bytes bytes) and the exponents of its rows ([n_aux_pad] ints)
 // come from launch_chi0_digits; dtab is the FP64 table; `work` (128-byte aligned) holds the digits of D O in chunks, at least
 // chi0_fixed_work_bytes(n_ov_pad, 128) bytes. Returns the launches, -1 on a launch error, -2 if unsupported.
-constexpr int kFixedMinAux = 64;
+// Sizes from which on the digits are the faster form (the SIMT build's 64 x 64 tiles run on after one another's k, the digits' cost
+// hardly depends on it up to there). Measured at N_aux 64 .. 416, 1 to 608 frequencies: N_ov 126 0.32 .. 0.91 of the SIMT build's time, 96
+// 0.42 .. 1.20, 65 0.5 .. 1.4, 8 1.8 .. 5.8. N_aux below 64 leaves half of every 128-row tile empty.
+constexpr int kFixedMinAux = 64, kFixedMinOv = 112;
 size_t chi0_fixed_digits_bytes(int n_aux_pad, int n_ov_pad);
 size_t chi0_fixed_work_bytes(int n_ov_pad, long long rows);
 bool chi0_fixed_shape(int n_aux, long long n_ov);  // the sizes it takes
