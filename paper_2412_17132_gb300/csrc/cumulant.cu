@@ -37,7 +37,7 @@ namespace {
 // Points next to zero (a window's rounding error, 1.1e-16 where 0 was meant), |w_j| t_max <= 2^-10, stay out of the blocks and
 // are added time by time as the direct sum adds them, up to MAXN of them; a core with more, or whose other coefficients sum
 // to more than 2^30, takes the direct sum. Measured (n_t = 2^16), the whole spectrum with the direct
-// sum below and with this: 6.66 and 0.154 ms for one core at 400 points, 26.5 and 0.831 ms for 22 cores.
+// sum below and with this: 6.66 and 0.156 ms for one core at 400 points, 26.5 and 0.856 ms for 22 cores.
 constexpr int NP = 32;       // Chebyshev nodes of a block, NH of them positive
 constexpr int NH = NP / 2;
 constexpr int MAXB = 1024;   // times per block, a power of two in NP .. MAXB
@@ -409,7 +409,7 @@ __device__ __forceinline__ double2 half_input(const double2* __restrict__ g, int
 // 2^LR-point Stockham pass of the half-length transform with span p (1, 2^LR, ...): LR radix-2 levels in registers, so a
 // transform of 2^15 points takes four passes over memory and four launches. FIRST forms Z from g, LAST writes
 // the spectrum: A on ascending nu, o = 0 <-> the most negative. 22 transforms for n_t = 2^16: 134 us (FP64
-// instructions and L2) against 221 us for one full-length radix-2 level per launch; the whole spectrum 0.935 -> 0.831 ms,
+// instructions and L2) against 221 us for one full-length radix-2 level per launch; the whole spectrum 0.935 -> 0.831 ms (blocks as then),
 // and for one core, where 18 launches became 5, 0.164 -> 0.154 ms.
 template <int LR, bool FIRST, bool LAST>
 __global__ void __launch_bounds__(64) stockham_pass_kernel(const double2* __restrict__ x, double2* __restrict__ y, int n, int p,
